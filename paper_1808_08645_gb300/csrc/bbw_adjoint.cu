@@ -348,6 +348,7 @@ bbw::StageParams<real> stage_params(bbw_solver* s, const void* qin, void* qout, 
   P.tau_p = real(s->tau_p);
   P.tau_u = real(s->tau_u);
   P.status = s->d_status;
+  bbw::set_lane<bbw::StageParams<real>, real>(s, P);
   return P;
 }
 
@@ -386,6 +387,8 @@ bbw_status adjoint_stage(bbw_solver* s, AdjointData* a, const void* vbr, int sta
   Q.G = s->G;
   Q.a = stage == 4 ? real(0) : real(ca[stage + 1]);
   Q.b = real(cb[stage]);
+  Q.lane = s->lane;
+  for (int j = 0; j <= s->N; ++j) Q.cs[j] = real(s->cj[j]);
   BBW_CUDA(s->ops->launch_adj_pre(s->M, s->prec == 64, &Q, s->grid_stage, st));
   // kap -= dt |D| A_{-tau}(y)
   bbw::StageParams<real> P = stage_params<real>(s, a->yi, a->kap, a->kap);

@@ -274,7 +274,7 @@ void free_solver(bbw_solver* s) {
   bbw::free_adjoint(s);
   for (void* p : {s->q[0], s->q[1], s->res, s->d_c2, s->d_geom, static_cast<void*>(s->d_conn), s->d_src,
                   static_cast<void*>(s->d_src_groups), static_cast<void*>(s->d_src_slots),
-                  static_cast<void*>(s->d_src_ser), static_cast<void*>(s->d_src_amp), s->d_stage,
+                  static_cast<void*>(s->d_src_ser), static_cast<void*>(s->d_src_amp), s->d_stage, s->d_rhs,
                   static_cast<void*>(s->d_perm),
                   static_cast<void*>(s->d_inv),
                   static_cast<void*>(s->d_status)})
@@ -503,6 +503,7 @@ bbw_status launch_stage(bbw_solver* s, int stage, double dt) {
   bbw::set_stage_sources<bbw::StageParams<real>, real>(s, P, s->steps, stage, true);
   P.status = s->d_status;
   P.vout = static_cast<real*>(s->vout);
+  bbw::set_lane<bbw::StageParams<real>, real>(s, P);
   BBW_CUDA(s->ops->launch_stage(s->M, s->prec == 64, &P, s->grid_stage, s->stream));
   s->cur = 1 - s->cur;
   s->stages += 1;
@@ -769,6 +770,8 @@ bbw_status bbw::create_solver(int64_t nverts, const double* vxyz, int64_t K, con
   }
   int team = 0, gpc = 1;
   s->ops->launch_shape(M, precision == 64, &team, &s->V, &gpc);
+  s->lane = s->ops->use_lane(M, precision == 64, K);
+  if (s->lane) s->V = 1;
   s->G = (K + s->V - 1) / s->V;
   const int64_t tiles = (s->G + gpc - 1) / gpc;
   s->grid_stage = int(std::min<int64_t>(tiles, int64_t(std::max(1, s->op->per_sm_stage)) * num_sms()));
@@ -783,6 +786,8 @@ bbw_status bbw::create_solver(int64_t nverts, const double* vxyz, int64_t K, con
             alloc(&s->res, s->nstate_internal() * rs) && alloc(&s->d_c2, ng * s->Mp * rs) &&
             alloc(&s->d_geom, ng * 9 * rs) && alloc(reinterpret_cast<void**>(&s->d_conn), ng * 16) &&
             alloc(reinterpret_cast<void**>(&s->d_status), 16);
+  const size_t nrhs = s->lane ? s->ops->lane_scratch(precision == 64, K) : 0;
+  ok = ok && (!nrhs || alloc(&s->d_rhs, nrhs * rs));
   if (!ok) {
     std::string msg = std::string("device allocation failed: ") + cudaGetErrorString(cudaGetLastError());
     free_solver(s);

@@ -161,6 +161,7 @@ bbw_status launch_bucket_step(bbw_batch* b, bbw_batch::Bucket& k, double dt, cud
     P.step_host = 0;
     P.stage = stage;
     P.status = s->d_status;
+    bbw::set_lane<bbw::StageParams<real>, real>(s, P);
     // autotuner trials step with dt = 0 (no per-group dt) but keep the
     // budgets, so that finished instances stay untouched (residual included)
     if (!b->trial) P.dt_group = static_cast<const real*>(k.d_dtg);
@@ -365,6 +366,11 @@ bbw_status bbw_batch_create(int n, const int64_t* nverts, const double* const* v
     k.members = ids;
     int team = 0, V = 1, gpc = 1;
     bbw::ops_for(deg)->launch_shape(M, precision == 64, &team, &V, &gpc);
+    // the bucket's kernels go by its size (they give the same bits as a solo
+    // solver's); V = 1 with the tile kernels. Group padding only adds elements.
+    int64_t total = 0;
+    for (int i : ids) total += K[i];
+    if (bbw::ops_for(deg)->use_lane(M, precision == 64, total)) V = 1;
     // disjoint union, every instance starting on a group boundary
     std::vector<double> xyz;
     std::vector<int64_t> tets;

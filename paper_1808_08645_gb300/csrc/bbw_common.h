@@ -44,6 +44,9 @@ constexpr int kPerm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 
 // or -1 on a wall. Limits the mesh to 2^26 elements.
 constexpr int64_t kMaxElements = int64_t(1) << 26;
 
+// rows of a block of 32 elements of the lane kernels' geometry (bbw_solver.h)
+constexpr int kLaneGeom = 13;
+
 // Packed stencil words. A one-degree reduction (E^n_{n-1})^T produces output
 // beta (degree n-1) from inputs beta + e_m (degree n) at
 //   base, base + 1, base + dk, base + dl,   base = idx3(n, j, k, l),

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <array>
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <utility>
@@ -75,6 +76,8 @@ struct bbw_solver {
   unsigned int* d_status = nullptr;
   void* pinned = nullptr;
   size_t pinned_bytes = 0;
+  bool lane = false;        // the tile kernels (one element per lane): V = 1
+  void* d_rhs = nullptr;    // their p bracket [K][Np]
   void* d_stage = nullptr;  // FP64 user-layout staging of host state transfers
   size_t d_stage_bytes = 0;
   int cur = 0;
@@ -153,6 +156,32 @@ void set_stage_sources(const bbw_solver* s, P_t& P, int64_t step, int stage, boo
   P.step_dev = nullptr;
   P.step_host = step;
   P.stage = stage;
+}
+
+// Which kernels a launch of solver s runs, and their scratch and constants.
+template <typename P_t, typename real>
+void set_lane(const bbw_solver* s, P_t& P) {
+  P.lane = s->lane;
+  P.rhs = static_cast<real*>(s->d_rhs);
+  for (int j = 0; j <= s->N; ++j) P.cs[j] = real(s->cj[j]);
+}
+
+// Geometry of the kernels with one element per lane, [ceil(K / 32)][13][32]:
+// d lambda_m / d x_i (m = 1..3), then 1 / |grad lambda_f| (f = 0..3).
+inline size_t lane_geometry_values(int64_t K) { return size_t((K + 31) / 32) * 32 * kLaneGeom; }
+template <typename real>
+std::vector<real> lane_geometry_rows(const bbw_solver* s) {
+  std::vector<real> h(lane_geometry_values(s->K));
+  for (size_t e = 0; e < h.size() / kLaneGeom; ++e) {
+    double g[12] = {-1, -1, -1, 1, 0, 0, 0, 1, 0, 0, 0, 1};  // padding: the unit tetrahedron
+    if (int64_t(e) < s->K)
+      for (int c = 0; c < 12; ++c) g[c] = s->grad[size_t(s->user(int64_t(e))) * 12 + c];
+    real* o = &h[e / 32 * 32 * kLaneGeom + e % 32];
+    for (int c = 0; c < 9; ++c) o[c * 32] = real(g[3 + c]);
+    for (int f = 0; f < 4; ++f)
+      o[(9 + f) * 32] = real(1.0 / std::sqrt(g[3 * f] * g[3 * f] + g[3 * f + 1] * g[3 * f + 1] + g[3 * f + 2] * g[3 * f + 2]));
+  }
+  return h;
 }
 
 }  // namespace bbw

@@ -90,6 +90,11 @@ struct StageParams {
   // the sources) is left as it is: q_out = q_in, res untouched.
   const real* __restrict__ dt_group = nullptr;     // [G]
   const int64_t* __restrict__ steps_group = nullptr;  // [G]
+  // the tile kernels (bbw_tile.cuh, layout of V = 1): lane is set; rhs the p
+  // bracket between the tile and the projection kernel [G][Np]; cs the c_j
+  bool lane = false;
+  real* __restrict__ rhs = nullptr;
+  real cs[kMaxN + 1] = {};
 };
 
 // One stage of the discrete adjoint before its spatial operator, in the
@@ -107,6 +112,8 @@ struct AdjPreParams {
   const void* __restrict__ tables;
   int64_t G;
   real a, b;
+  bool lane = false;              // the kernel with one element per lane (bbw_tile.cuh, layout of V = 1)
+  real cs[kMaxN + 1] = {};        // its projection constants c_j
 };
 
 template <typename real>

@@ -4,8 +4,11 @@
 
 #include <new>
 
+#include <cstddef>
+
 #include "bbw_ops.h"
 #include "bbw_stage.cuh"
+#include "bbw_tile.cuh"
 
 #ifndef BBW_N
 #error "define BBW_N before including bbw_stage_inst.cuh"
@@ -42,6 +45,34 @@ constexpr auto adj_pre_fn() {
   return adj_pre_kernel<kN, M, real, Shape<real>::T, Shape<real>::V, kGC<M, real>>;
 }
 
+// The tile kernels (bbw_tile.cuh) run solvers of at least kLaneMin elements,
+// N <= 6 in FP32 and N <= 5 in FP64; the team kernels (bbw_stage.cuh) the rest
+// (the same bits either way). A tile has 32 elements, so small meshes leave
+// SMs idle, and a warp's chain of work is longer than a team's. Stage times in
+// us, tile / team, M = 2, at 384 / 4,374 / 24,576 / 82,944 elements, FP32:
+//   N = 1  6.3/6.6, 7.3/8.3, 10/10, 20/27     N = 2  10/8.3, 10/8.4, 15/21, 34/47
+//   N = 3  12/10, 13/11, 20/31, 51/84         N = 4  17/20, 18/21, 42/51, 110/146
+//   N = 5  19/27, 20/29, 44/75, 145/219       N = 6  27/21, 29/21, 100/105, 270/302
+// (10,368 elements: N = 2 12.0/12.5, N = 3 14/18, N = 6 56/54; N = 7 at 82,944
+// 456/412, and N >= 8 does not fit), and FP64 at 384 / 6,000 / 16,464 elements:
+//   N = 1  18/27, 23/29, 37/47      N = 2  38/35, 53/62, 89/121    N = 3  60/37, 91/96, 156/245
+//   N = 4  111/120, 152/236, 299/466               N = 5  187/94, 267/275, 448/636
+template <typename real>
+constexpr bool kLane = kN <= (sizeof(real) == 4 ? 6 : 5);
+template <typename real>
+constexpr int64_t kLaneMin = sizeof(real) == 4 ? (kN == 2 ? 10000 : kN == 3 ? 9000 : kN == 6 ? 16000 : 0)
+                                               : (kN == 2 || kN == 3 ? 5000 : kN == 5 ? 6000 : 0);
+// The projection of p runs in the tile kernel where its levels fit the
+// registers (N <= 5, FP64 4); at N = 6 one warp of four would work on it for
+// longer than the rest of the tile takes (291 us fused, 270 apart).
+template <typename real>
+constexpr bool kFuseProjection = kN <= (sizeof(real) == 4 ? 5 : 4);
+template <typename real>
+constexpr int kStageMode = kFuseProjection<real> ? kFused : kBracket;
+template <int M, typename real, int MODE>
+constexpr auto tile_fn() {
+  return acoustic_tile_kernel<kN, MODE == kFused ? M : 0, real, MODE>;  // only the fused kernel depends on M
+}
 
 template <typename F>
 auto dispatch(int M, bool dbl, F&& f) {
@@ -93,18 +124,28 @@ void face_maps(int* fidx, int* nidx) {
   delete t;
 }
 
+template <typename K>
+cudaError_t allow_smem(K kernel, int bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 cudaError_t prepare(int M, bool dbl, int* per_sm_stage, int* per_sm_wadg) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
     auto ks = stage_fn<MM, real>();
     auto kw = wadg_fn<MM, real>();
-    cudaError_t err = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(kw, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(spatial_fn<MM, real>(), cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(adj_pre_fn<MM, real>(), cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    cudaError_t err = allow_smem(ks, C::SMEM);
+    if (err == cudaSuccess) err = allow_smem(kw, C::SMEM);
+    if (err == cudaSuccess) err = allow_smem(spatial_fn<MM, real>(), C::SMEM);
+    if (err == cudaSuccess) err = allow_smem(adj_pre_fn<MM, real>(), C::SMEM);
+    if constexpr (kLane<real>) {
+      using PC = ProjectShape<kN, MM, real>;
+      if (err == cudaSuccess) err = allow_smem(tile_fn<MM, real, kStageMode<real>>(), TileCfg<kN, real>::SMEM);
+      if (err == cudaSuccess) err = allow_smem(tile_fn<MM, real, kSpatial>(), TileCfg<kN, real>::SMEM);
+      if (err == cudaSuccess) err = allow_smem(lane_adj_pre_kernel<kN, MM, real>, PC::SMEM);
+      if constexpr (!kFuseProjection<real>)
+        if (err == cudaSuccess) err = allow_smem(acoustic_project_kernel<kN, MM, real>, PC::SMEM);
+    }
     if (err != cudaSuccess) return err;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm_stage, ks, C::THREADS, C::SMEM);
     if (err != cudaSuccess) return err;
@@ -112,11 +153,39 @@ cudaError_t prepare(int M, bool dbl, int* per_sm_stage, int* per_sm_wadg) {
   });
 }
 
+// Warps per CTA of a kernel with one warp per 32 elements: one where the warps
+// would not fill two CTAs on each of the 152 SMs.
+template <typename C>
+int lane_warps(int64_t G) {
+  return (G + 31) / 32 < int64_t(2 * 152) * C::WARPS ? 1 : C::WARPS;
+}
+
+template <int M, typename real, int MODE>
+void launch_tiles(const StageParams<real>& P, cudaStream_t s) {
+  using Tab = Tables<kN, M, real>;
+  constexpr size_t at = offsetof(Tab, fidx);  // fidx and nidx, one after the other
+  static_assert(at % 4 == 0 && offsetof(Tab, nidx) == at + sizeof(uint16_t) * 4 * np2(kN), "face tables");
+  tile_fn<M, real, MODE>()<<<unsigned((P.G + 31) / 32), 128, TileCfg<kN, real>::SMEM, s>>>(
+      P, reinterpret_cast<const uint32_t*>(static_cast<const char*>(P.tables) + at));
+}
+
 cudaError_t launch_stage(int M, bool dbl, const void* params, int grid, cudaStream_t s) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    stage_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(
-        *static_cast<const StageParams<real>*>(params));
+    const auto& P = *static_cast<const StageParams<real>*>(params);
+    if constexpr (kLane<real>) {
+      if (P.lane) {
+        launch_tiles<MM, real, kStageMode<real>>(P, s);
+        if constexpr (!kFuseProjection<real>) {
+          using PC = ProjectShape<kN, MM, real>;
+          const int w = lane_warps<PC>(P.G);
+          acoustic_project_kernel<kN, MM, real>
+              <<<unsigned((P.G + 32 * w - 1) / (32 * w)), 32 * w, w * PC::WARP_BYTES, s>>>(P);
+        }
+        return cudaGetLastError();
+      }
+    }
+    stage_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
     return cudaGetLastError();
   });
 }
@@ -124,8 +193,14 @@ cudaError_t launch_stage(int M, bool dbl, const void* params, int grid, cudaStre
 cudaError_t launch_spatial(int M, bool dbl, const void* params, int grid, cudaStream_t s) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    spatial_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(
-        *static_cast<const StageParams<real>*>(params));
+    const auto& P = *static_cast<const StageParams<real>*>(params);
+    if constexpr (kLane<real>) {
+      if (P.lane) {
+        launch_tiles<MM, real, kSpatial>(P, s);
+        return cudaGetLastError();
+      }
+    }
+    spatial_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
     return cudaGetLastError();
   });
 }
@@ -142,9 +217,27 @@ cudaError_t launch_wadg(int M, bool dbl, const void* params, int grid, cudaStrea
 cudaError_t launch_adj_pre(int M, bool dbl, const void* params, int grid, cudaStream_t s) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    adj_pre_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(*static_cast<const AdjPreParams<real>*>(params));
+    const auto& P = *static_cast<const AdjPreParams<real>*>(params);
+    if constexpr (kLane<real>) {
+      if (P.lane) {
+        using PC = ProjectShape<kN, MM, real>;
+        const int w = lane_warps<PC>(P.G);
+        lane_adj_pre_kernel<kN, MM, real>
+            <<<4 * unsigned((P.G + 32 * w - 1) / (32 * w)), 32 * w, w * PC::WARP_BYTES, s>>>(P);
+        return cudaGetLastError();
+      }
+    }
+    adj_pre_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
     return cudaGetLastError();
   });
+}
+
+bool use_lane(int M, bool dbl, int64_t K) {
+  return dispatch(M, dbl, [&]<int MM, typename real>() { return kLane<real> && K >= kLaneMin<real>; });
+}
+
+size_t lane_scratch(bool dbl, int64_t K) {
+  return (dbl ? kFuseProjection<double> : kFuseProjection<float>) ? 0 : size_t(K) * np3(kN);
 }
 
 }  // namespace
@@ -154,7 +247,7 @@ cudaError_t launch_adj_pre(int M, bool dbl, const void* params, int grid, cudaSt
 const KernelOps& BBW_CAT(ops_n, BBW_N)() {
   static const KernelOps ops = {&tables_size,  &build,          &face_maps,    &prepare,
                                 &launch_stage, &launch_wadg,    &launch_shape, &launch_spatial,
-                                &check_tables, &launch_adj_pre};
+                                &check_tables, &launch_adj_pre, &use_lane,     &lane_scratch};
   return ops;
 }
 
