@@ -30,6 +30,9 @@ struct bbw_elastic {
   void* d_media = nullptr;  // [G][3][Mp][V]
   void* d_geom = nullptr;   // [G][9][V]
   int32_t* d_conn = nullptr;  // [G][4][V]
+  void* d_flux = nullptr;   // scratch of the kernels with one element per lane: face fluxes,
+  void* d_rhs = nullptr;    // brackets [K][10][Np]
+  double cs[bbw::kMaxN + 1] = {};  // constants of their projections
   void* d_stage = nullptr;  // FP64 user-layout staging of host state transfers
   std::vector<double> media;  // [3][K][Mp], caller's element order
   int cur = 0;
@@ -86,7 +89,7 @@ int conv_blocks(size_t n) { return int(std::min<size_t>((n + 255) / 256, size_t(
 
 void free_elastic(bbw_elastic* s) {
   if (!s) return;
-  for (void* p : {s->q[0], s->q[1], s->res, s->d_media, s->d_geom, static_cast<void*>(s->d_conn), s->d_stage})
+  for (void* p : {s->q[0], s->q[1], s->res, s->d_media, s->d_geom, static_cast<void*>(s->d_conn), s->d_flux, s->d_rhs, s->d_stage})
     if (p) cudaFree(p);
   if (s->m) bbw_destroy(s->m);
   delete s;
@@ -111,6 +114,10 @@ template <typename real>
 bbw_status upload_mesh(bbw_elastic* s) {
   bbw_solver* m = s->m;
   const int V = s->V;
+  if (s->d_flux) {
+    const std::vector<real> rows = bbw::lane_geometry_rows<real>(m);
+    BBW_CUDA(cudaMemcpy(s->d_geom, rows.data(), rows.size() * sizeof(real), cudaMemcpyHostToDevice));
+  } else {
   // geometry [G][9][V]: d lambda_m / d x for m = 1..3; padding: the unit tetrahedron
   std::vector<double> g9(size_t(m->K) * 9);
   for (int64_t e = 0; e < m->K; ++e)
@@ -122,6 +129,7 @@ bbw_status upload_mesh(bbw_elastic* s) {
         h[(size_t(e / V) * 9 + c) * V + size_t(e % V)] =
             real(e < m->K ? g9[size_t(m->user(e)) * 9 + c] : (c % 4 == 0 ? 1.0 : 0.0));
     BBW_CUDA(cudaMemcpy(s->d_geom, h.data(), h.size() * sizeof(real), cudaMemcpyHostToDevice));
+  }
   }
   // connectivity [G][4][V]: (internal neighbour slot << 5) | (its face << 3) | orientation; -1: wall
   std::vector<int32_t> conn(size_t(s->G) * 4 * V, -1);
@@ -154,6 +162,9 @@ bbw_status launch(bbw_elastic* s, int stage, double dt) {
   P.tau_v = real(s->tau_v);
   P.tau_s = real(s->tau_s);
   P.status = m->d_status;
+  P.flux = static_cast<real*>(s->d_flux);
+  P.rhs = static_cast<real*>(s->d_rhs);
+  for (int j = 0; j <= m->N; ++j) P.cs[j] = real(s->cs[j]);
   BBW_CUDA(s->ops->launch(m->M, m->prec == 64, &P, s->grid, m->stream));
   s->cur = 1 - s->cur;
   s->stages += 1;
@@ -228,7 +239,10 @@ bbw_status bbw_elastic_create(int64_t nverts, const double* vxyz, int64_t K, con
   }
   s->ops = bbw::elastic_ops_for(N);
   int team = 0, gpc = 1, per_sm = 0;
-  s->ops->shape(M, precision == 64, &team, &s->V, &gpc);
+  int width = 1;
+  size_t nflux = 0, nrhs = 0;
+  s->ops->shape(M, precision == 64, &team, &width, &gpc);
+  s->V = s->ops->layout(M, precision == 64, K, &nflux, &nrhs);
   cudaError_t err = s->ops->prepare(M, precision == 64, &per_sm);
   if (err != cudaSuccess) {
     free_elastic(s);
@@ -239,6 +253,7 @@ bbw_status bbw_elastic_create(int64_t nverts, const double* vxyz, int64_t K, con
   s->grid = int(std::min<int64_t>(tiles, int64_t(std::max(1, per_sm)) * sm_count()));
   double c[5];
   bbw_lsrk_coeffs(s->rk_a, s->rk_b, c);
+  s->ops->projection_scale(M, m->cj, s->cs);
   const size_t rs = s->rsz();
   const size_t ng = size_t(s->G) * s->V;
   auto alloc = [&](void** p, size_t bytes) {
@@ -246,8 +261,9 @@ bbw_status bbw_elastic_create(int64_t nverts, const double* vxyz, int64_t K, con
   };
   const bool ok = alloc(&s->q[0], s->ninternal() * rs) && alloc(&s->q[1], s->ninternal() * rs) &&
                   alloc(&s->res, s->ninternal() * rs) && alloc(&s->d_media, ng * 3 * m->Mp * rs) &&
-                  alloc(&s->d_geom, ng * 9 * rs) && alloc(reinterpret_cast<void**>(&s->d_conn), ng * 16) &&
-                  alloc(&s->d_stage, s->nuser() * 8);
+                  alloc(&s->d_geom, (nflux ? bbw::lane_geometry_values(K) : ng * 9) * rs) && alloc(reinterpret_cast<void**>(&s->d_conn), ng * 16) &&
+                  alloc(&s->d_stage, s->nuser() * 8) &&
+                  (!nflux || alloc(&s->d_flux, nflux * rs)) && (!nrhs || alloc(&s->d_rhs, nrhs * rs));
   if (!ok) {
     std::string msg = std::string("device allocation failed: ") + cudaGetErrorString(cudaGetLastError());
     free_elastic(s);

@@ -47,6 +47,13 @@ struct ElasticParams {
   real a, b, dt;
   real tau_v, tau_s;
   unsigned int* status;  // bit 0: non-finite output; bit 1 (checked build): index out of range
+  // one element per lane (bbw_elastic_lane.cuh, V = 1): the fluxes at the face
+  // nodes [ceil(G / 32)][6][4][Nfp][32]; the brackets of the ten field tasks
+  // as power coefficients [G][10][Np] (fused kernels use the tenth alone, for
+  // the projected trace); the constants of the projection
+  real* __restrict__ flux = nullptr;
+  real* __restrict__ rhs = nullptr;
+  real cs[kMaxN + 1] = {};
 };
 
 template <int N, typename real>
