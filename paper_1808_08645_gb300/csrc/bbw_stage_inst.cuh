@@ -54,13 +54,15 @@ constexpr auto adj_pre_fn() {
 //   N = 3  12/10, 13/11, 20/31, 51/84         N = 4  17/20, 18/21, 42/51, 110/146
 //   N = 5  19/27, 20/29, 44/75, 145/219       N = 6  27/21, 29/21, 100/105, 270/302
 // (10,368 elements: N = 2 12.0/12.5, N = 3 14/18, N = 6 56/54; N = 7 at 82,944
-// 456/412, and N >= 8 does not fit), and FP64 at 384 / 6,000 / 16,464 elements:
+// 456/412, and N >= 8 does not fit). N = 6 gains least, and at M = 0 nothing
+// at 24,576 (92/91) and 256/262 at 82,944; a last wave in between can cost 5 %,
+// so it switches above those. FP64 at 384 / 6,000 / 16,464 elements:
 //   N = 1  18/27, 23/29, 37/47      N = 2  38/35, 53/62, 89/121    N = 3  60/37, 91/96, 156/245
 //   N = 4  111/120, 152/236, 299/466               N = 5  187/94, 267/275, 448/636
 template <typename real>
 constexpr bool kLane = kN <= (sizeof(real) == 4 ? 6 : 5);
 template <typename real>
-constexpr int64_t kLaneMin = sizeof(real) == 4 ? (kN == 2 ? 10000 : kN == 3 ? 9000 : kN == 6 ? 16000 : 0)
+constexpr int64_t kLaneMin = sizeof(real) == 4 ? (kN == 2 ? 10000 : kN == 3 ? 9000 : kN == 6 ? 80000 : 0)
                                                : (kN == 2 || kN == 3 ? 5000 : kN == 5 ? 6000 : 0);
 // The projection of p runs in the tile kernel where its levels fit the
 // registers (N <= 5, FP64 4); at N = 6 one warp of four would work on it for

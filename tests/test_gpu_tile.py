@@ -30,7 +30,7 @@ def case(n, N, M, seed):
 
 
 # hexes per side of three instances: two small ones, and one that takes the bucket over its degree's switching size
-@pytest.mark.parametrize("prec,N,ns", [(32, 2, (3, 5, 12)), (32, 3, (3, 5, 12)), (32, 6, (3, 5, 14)), (64, 2, (3, 5, 9)),
+@pytest.mark.parametrize("prec,N,ns", [(32, 2, (3, 5, 12)), (32, 3, (3, 5, 12)), (32, 6, (3, 5, 24)), (64, 2, (3, 5, 9)),
                                        (64, 3, (3, 5, 9)), (64, 5, (3, 5, 10))])
 @pytest.mark.parametrize("M", [0, 1, 3])
 def test_tile_and_team_bits(prec, N, ns, M):
