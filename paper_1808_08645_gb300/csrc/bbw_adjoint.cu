@@ -332,8 +332,8 @@ void free_run(AdjointData* a, bool release = false) {
 
 // The solver's launch parameters for a stage on explicit buffers.
 template <typename real>
-bbw::StageParams<real> stage_params(bbw_solver* s, const void* qin, void* qout, void* res) {
-  bbw::StageParams<real> P;
+bbw::LaneStageParams<real> stage_params(bbw_solver* s, const void* qin, void* qout, void* res) {
+  bbw::LaneStageParams<real> P;
   P.qin = static_cast<const real*>(qin);
   P.qout = static_cast<real*>(qout);
   P.res = static_cast<real*>(res);
@@ -348,7 +348,7 @@ bbw::StageParams<real> stage_params(bbw_solver* s, const void* qin, void* qout, 
   P.tau_p = real(s->tau_p);
   P.tau_u = real(s->tau_u);
   P.status = s->d_status;
-  bbw::set_lane<bbw::StageParams<real>, real>(s, P);
+  bbw::set_lane<bbw::LaneStageParams<real>, real>(s, P);
   return P;
 }
 
@@ -359,11 +359,11 @@ bbw_status forward_stage(bbw_solver* s, const void* qin, void* qout, void* res, 
                          void* vout) {
   double ca[5], cb[5];
   bbw_lsrk_coeffs(ca, cb, nullptr);
-  bbw::StageParams<real> P = stage_params<real>(s, qin, qout, res);
+  bbw::LaneStageParams<real> P = stage_params<real>(s, qin, qout, res);
   P.a = real(ca[stage]);
   P.b = real(cb[stage]);
   P.dt = real(dt);
-  bbw::set_stage_sources<bbw::StageParams<real>, real>(s, P, step, stage, true);
+  bbw::set_stage_sources<bbw::LaneStageParams<real>, real>(s, P, step, stage, true);
   P.vout = static_cast<real*>(vout);
   BBW_CUDA(s->ops->launch_stage(s->M, s->prec == 64, &P, s->grid_stage, s->stream));
   return BBW_OK;
@@ -377,7 +377,7 @@ bbw_status adjoint_stage(bbw_solver* s, AdjointData* a, const void* vbr, int sta
   cudaStream_t st = s->stream;
   // rho_t = a_{s+1} rho + b_s kap (rho holds rho_t of the stage after; at the
   // last stage of a step the incoming res cotangent is zero, a_0 = 0); y
-  bbw::AdjPreParams<real> Q;
+  bbw::LaneAdjPreParams<real> Q;
   Q.rho = static_cast<real*>(a->rho);
   Q.kap = static_cast<const real*>(a->kap);
   Q.c2 = static_cast<const real*>(s->d_c2);
@@ -391,12 +391,12 @@ bbw_status adjoint_stage(bbw_solver* s, AdjointData* a, const void* vbr, int sta
   for (int j = 0; j <= s->N; ++j) Q.cs[j] = real(s->cj[j]);
   BBW_CUDA(s->ops->launch_adj_pre(s->M, s->prec == 64, &Q, s->grid_stage, st));
   // kap -= dt |D| A_{-tau}(y)
-  bbw::StageParams<real> P = stage_params<real>(s, a->yi, a->kap, a->kap);
+  bbw::LaneStageParams<real> P = stage_params<real>(s, a->yi, a->kap, a->kap);
   P.tau_p = real(-s->tau_p);
   P.tau_u = real(-s->tau_u);
   P.dt = real(dt);
   P.accumulate = 1;
-  bbw::set_stage_sources<bbw::StageParams<real>, real>(s, P, 0, stage, false);
+  bbw::set_stage_sources<bbw::LaneStageParams<real>, real>(s, P, 0, stage, false);
   BBW_CUDA(s->ops->launch_spatial(s->M, s->prec == 64, &P, s->grid_stage, st));
   // gc += dt rho_t,p^T T_beta v
   const size_t ops = (size_t(2) * s->Np + size_t(kGradWarps) * s->Mp) * 32 * sizeof(real);  // staged operands, partials

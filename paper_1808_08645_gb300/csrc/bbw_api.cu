@@ -486,7 +486,7 @@ bbw_status upload_geometry(bbw_solver* s) {
 
 template <typename real>
 bbw_status launch_stage(bbw_solver* s, int stage, double dt) {
-  bbw::StageParams<real> P;
+  bbw::LaneStageParams<real> P;
   P.qin = static_cast<const real*>(s->q[s->cur]);
   P.qout = static_cast<real*>(s->q[1 - s->cur]);
   P.res = static_cast<real*>(s->res);
@@ -500,10 +500,10 @@ bbw_status launch_stage(bbw_solver* s, int stage, double dt) {
   P.dt = real(dt);
   P.tau_p = real(s->tau_p);
   P.tau_u = real(s->tau_u);
-  bbw::set_stage_sources<bbw::StageParams<real>, real>(s, P, s->steps, stage, true);
+  bbw::set_stage_sources<bbw::LaneStageParams<real>, real>(s, P, s->steps, stage, true);
   P.status = s->d_status;
   P.vout = static_cast<real*>(s->vout);
-  bbw::set_lane<bbw::StageParams<real>, real>(s, P);
+  bbw::set_lane<bbw::LaneStageParams<real>, real>(s, P);
   BBW_CUDA(s->ops->launch_stage(s->M, s->prec == 64, &P, s->grid_stage, s->stream));
   s->cur = 1 - s->cur;
   s->stages += 1;

@@ -136,7 +136,7 @@ bbw_status launch_bucket_step(bbw_batch* b, bbw_batch::Bucket& k, double dt, cud
   bbw_solver* s = k.s;
   int cur = b->cur;
   for (int stage = 0; stage < 5; ++stage) {
-    bbw::StageParams<real> P;
+    bbw::LaneStageParams<real> P;
     P.qin = static_cast<const real*>(s->q[cur]);
     P.qout = static_cast<real*>(s->q[1 - cur]);
     P.res = static_cast<real*>(s->res);
@@ -161,7 +161,7 @@ bbw_status launch_bucket_step(bbw_batch* b, bbw_batch::Bucket& k, double dt, cud
     P.step_host = 0;
     P.stage = stage;
     P.status = s->d_status;
-    bbw::set_lane<bbw::StageParams<real>, real>(s, P);
+    bbw::set_lane<bbw::LaneStageParams<real>, real>(s, P);
     // autotuner trials step with dt = 0 (no per-group dt) but keep the
     // budgets, so that finished instances stay untouched (residual included)
     if (!b->trial) P.dt_group = static_cast<const real*>(k.d_dtg);

@@ -147,7 +147,7 @@ bbw_status upload_mesh(bbw_elastic* s) {
 template <typename real>
 bbw_status launch(bbw_elastic* s, int stage, double dt) {
   bbw_solver* m = s->m;
-  bbw::ElasticParams<real> P;
+  bbw::LaneElasticParams<real> P;
   P.qin = static_cast<const real*>(s->q[s->cur]);
   P.qout = static_cast<real*>(s->q[1 - s->cur]);
   P.res = static_cast<real*>(s->res);

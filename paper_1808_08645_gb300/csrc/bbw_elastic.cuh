@@ -47,14 +47,24 @@ struct ElasticParams {
   real a, b, dt;
   real tau_v, tau_s;
   unsigned int* status;  // bit 0: non-finite output; bit 1 (checked build): index out of range
-  // one element per lane (bbw_elastic_lane.cuh, V = 1): the fluxes at the face
-  // nodes [ceil(G / 32)][6][4][Nfp][32]; the brackets of the ten field tasks
-  // as power coefficients [G][10][Np] (fused kernels use the tenth alone, for
-  // the projected trace); the constants of the projection
+};
+
+// What the kernels with one element per lane (bbw_elastic_lane.cuh, V = 1)
+// take besides; flux says which kernels run. It is apart from ElasticParams
+// because the team kernel's register allocation goes with the size of its
+// parameters (N = 6, M = 1: 41 us a stage at 1,296 elements with the fields in
+// one struct, 39 without).
+template <typename real>
+struct LaneElasticParams : ElasticParams<real> {
+  // the fluxes at the face nodes [ceil(G / 32)][6][4][Nfp][32]; the brackets of
+  // the ten field tasks as power coefficients [G][10][Np] (fused kernels use
+  // the tenth alone, for the projected trace); the constants of the projection
   real* __restrict__ flux = nullptr;
   real* __restrict__ rhs = nullptr;
   real cs[kMaxN + 1] = {};
 };
+static_assert(offsetof(ElasticParams<float>, status) + sizeof(void*) == sizeof(ElasticParams<float>),
+              "the team kernel's parameters hold nothing of the lane kernels'");
 
 template <int N, typename real>
 struct ElasticShape;

@@ -88,7 +88,7 @@ cudaError_t eprepare(int M, bool dbl, int* per_sm) {
 cudaError_t elaunch(int M, bool dbl, const void* params, int grid, cudaStream_t s) {
   return edispatch(M, dbl, [&]<int MM, typename real>() {
     using C = ECfg<MM, real>;
-    const auto& P = *static_cast<const ElasticParams<real>*>(params);
+    const auto& P = *static_cast<const LaneElasticParams<real>*>(params);
     if constexpr (kELane<real>) {
       if (P.flux) {
         using Tab = Tables<kN, MM, real>;

@@ -38,7 +38,7 @@ struct Elastic {
 };
 
 template <int N, typename real>
-__global__ void __launch_bounds__(kFluxThreads) elastic_flux_kernel(const ElasticParams<real> P,
+__global__ void __launch_bounds__(kFluxThreads) elastic_flux_kernel(const LaneElasticParams<real> P,
                                                                     const uint16_t* __restrict__ fidx,
                                                                     const uint16_t* __restrict__ nidx) {
   flux_tile<Elastic, N, real>(
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kFluxThreads) elastic_flux_kernel(const Elasti
 // The projected right-hand side of a field in the columns -> its RK update;
 // the trace task stores its projection instead. task as in Elastic::task.
 template <int N, typename real, int S>
-__device__ __forceinline__ void elastic_finish(const ElasticParams<real>& P, real* cols, int64_t e0, int ne, int lane,
+__device__ __forceinline__ void elastic_finish(const LaneElasticParams<real>& P, real* cols, int64_t e0, int ne, int lane,
                                                int task) {
   using Tile = WarpTile<np3(N), real>;
   constexpr int Np = np3(N);
@@ -107,7 +107,7 @@ __device__ __forceinline__ int elastic_weight(int task) { return task < 3 ? 0 : 
 // ten brackets go to P.rhs for elastic_project_kernel.
 template <int N, int M, typename real, bool FUSED, bool TRACE>
 __global__ void __launch_bounds__(FieldShape<N, real>::THREADS, N == 5 ? 2 : kFieldCtas<N>)
-    elastic_field_kernel(const ElasticParams<real> P) {
+    elastic_field_kernel(const LaneElasticParams<real> P) {
   using C = FieldShape<N, real>;
   using Tile = WarpTile<np3(N), real>;
   constexpr int Np = np3(N), Mp = np3(M), S = C::S;
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(FieldShape<N, real>::THREADS, N == 5 ? 2 : kFi
 // the fused elastic_field_kernel.
 template <int N, int M, typename real, bool TRACE>
 __global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS)
-    elastic_project_kernel(const ElasticParams<real> P) {
+    elastic_project_kernel(const LaneElasticParams<real> P) {
   using C = ProjectShape<N, M, real>;
   using Tile = WarpTile<np3(N), real>;
   constexpr int Np = np3(N), Mp = np3(M), S = C::S;

@@ -14,7 +14,7 @@ namespace bbw {
 struct ElasticOps {
   // set the shared-memory attribute, return CTAs per SM of the stage kernel
   cudaError_t (*prepare)(int M, bool dbl, int* ctas_per_sm);
-  // launch one stage; params points to ElasticParams<float|double>
+  // launch one stage; params points to LaneElasticParams<float|double>
   cudaError_t (*launch)(int M, bool dbl, const void* params, int grid, cudaStream_t s);
   // launch shape: lanes per group, elements per group, groups per CTA
   void (*shape)(int M, bool dbl, int* team, int* group_width, int* groups_per_cta);

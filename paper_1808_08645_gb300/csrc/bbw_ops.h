@@ -19,17 +19,17 @@ struct KernelOps {
   void (*face_maps)(int* fidx, int* nidx);
   // set the shared-memory attribute, return CTAs per SM for the stage / wadg kernel
   cudaError_t (*prepare)(int M, bool dbl, int* stage_ctas_per_sm, int* wadg_ctas_per_sm);
-  // launch one stage; params points to StageParams<float|double>
+  // launch one stage; params points to LaneStageParams<float|double>
   cudaError_t (*launch_stage)(int M, bool dbl, const void* params, int grid, cudaStream_t s);
   // launch the weight-adjusted update; params points to WadgParams<float|double>
   cudaError_t (*launch_wadg)(int M, bool dbl, const void* params, int grid, cudaStream_t s);
   // launch shape: lanes per group, elements per group, groups per CTA
   void (*launch_shape)(int M, bool dbl, int* team, int* group_width, int* groups_per_cta);
-  // launch the spatial operator alone (StageParams, output in qout)
+  // launch the spatial operator alone (LaneStageParams, output in qout)
   cudaError_t (*launch_spatial)(int M, bool dbl, const void* params, int grid, cudaStream_t s);
   // host-only: build the tables and check them against brute force (nullptr: all agree)
   const char* (*check_tables)(int M, bool dbl, const double* cj);
-  // launch the adjoint stage's pre-kernel; params points to AdjPreParams<float|double>
+  // launch the adjoint stage's pre-kernel; params points to LaneAdjPreParams<float|double>
   cudaError_t (*launch_adj_pre)(int M, bool dbl, const void* params, int grid, cudaStream_t s);
   // whether a solver of K elements runs the tile kernels (bbw_tile.cuh; the
   // launch entries do so when the parameters' lane is set)

@@ -43,6 +43,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cstddef>
+
 #include "bbw_common.h"
 
 namespace bbw {
@@ -90,11 +92,17 @@ struct StageParams {
   // the sources) is left as it is: q_out = q_in, res untouched.
   const real* __restrict__ dt_group = nullptr;     // [G]
   const int64_t* __restrict__ steps_group = nullptr;  // [G]
-  // the tile kernels (bbw_tile.cuh, layout of V = 1): lane is set; rhs the p
-  // bracket between the tile and the projection kernel [G][Np]; cs the c_j
+};
+
+// What the tile kernels (bbw_tile.cuh, layout of V = 1) take besides. The
+// launch entries get this struct; lane says which kernels run. It is apart
+// from StageParams because the team kernels' register allocation goes with the
+// size of their parameters.
+template <typename real>
+struct LaneStageParams : StageParams<real> {
   bool lane = false;
-  real* __restrict__ rhs = nullptr;
-  real cs[kMaxN + 1] = {};
+  real* __restrict__ rhs = nullptr;  // p bracket between the tile and the projection kernel [G][Np]
+  real cs[kMaxN + 1] = {};           // the c_j
 };
 
 // One stage of the discrete adjoint before its spatial operator, in the
@@ -112,9 +120,17 @@ struct AdjPreParams {
   const void* __restrict__ tables;
   int64_t G;
   real a, b;
-  bool lane = false;              // the kernel with one element per lane (bbw_tile.cuh, layout of V = 1)
-  real cs[kMaxN + 1] = {};        // its projection constants c_j
 };
+
+// The same for the kernel with one element per lane, as LaneStageParams.
+template <typename real>
+struct LaneAdjPreParams : AdjPreParams<real> {
+  bool lane = false;
+  real cs[kMaxN + 1] = {};  // its projection constants c_j
+};
+static_assert(offsetof(StageParams<float>, steps_group) + sizeof(void*) == sizeof(StageParams<float>) &&
+                  offsetof(AdjPreParams<double>, b) + sizeof(double) == sizeof(AdjPreParams<double>),
+              "the team kernels' parameters hold nothing of the lane kernels'");
 
 template <typename real>
 struct WadgParams {

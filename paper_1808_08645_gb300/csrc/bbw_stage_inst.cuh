@@ -163,7 +163,7 @@ int lane_warps(int64_t G) {
 }
 
 template <int M, typename real, int MODE>
-void launch_tiles(const StageParams<real>& P, cudaStream_t s) {
+void launch_tiles(const LaneStageParams<real>& P, cudaStream_t s) {
   using Tab = Tables<kN, M, real>;
   constexpr size_t at = offsetof(Tab, fidx);  // fidx and nidx, one after the other
   static_assert(at % 4 == 0 && offsetof(Tab, nidx) == at + sizeof(uint16_t) * 4 * np2(kN), "face tables");
@@ -174,7 +174,7 @@ void launch_tiles(const StageParams<real>& P, cudaStream_t s) {
 cudaError_t launch_stage(int M, bool dbl, const void* params, int grid, cudaStream_t s) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    const auto& P = *static_cast<const StageParams<real>*>(params);
+    const auto& P = *static_cast<const LaneStageParams<real>*>(params);
     if constexpr (kLane<real>) {
       if (P.lane) {
         launch_tiles<MM, real, kStageMode<real>>(P, s);
@@ -195,7 +195,7 @@ cudaError_t launch_stage(int M, bool dbl, const void* params, int grid, cudaStre
 cudaError_t launch_spatial(int M, bool dbl, const void* params, int grid, cudaStream_t s) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    const auto& P = *static_cast<const StageParams<real>*>(params);
+    const auto& P = *static_cast<const LaneStageParams<real>*>(params);
     if constexpr (kLane<real>) {
       if (P.lane) {
         launch_tiles<MM, real, kSpatial>(P, s);
@@ -219,7 +219,7 @@ cudaError_t launch_wadg(int M, bool dbl, const void* params, int grid, cudaStrea
 cudaError_t launch_adj_pre(int M, bool dbl, const void* params, int grid, cudaStream_t s) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    const auto& P = *static_cast<const AdjPreParams<real>*>(params);
+    const auto& P = *static_cast<const LaneAdjPreParams<real>*>(params);
     if constexpr (kLane<real>) {
       if (P.lane) {
         using PC = ProjectShape<kN, MM, real>;

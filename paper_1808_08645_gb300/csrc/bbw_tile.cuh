@@ -68,7 +68,7 @@ struct TileCfg {
 
 template <int N, int M, typename real, int MODE>
 __global__ void __launch_bounds__(128, TileCfg<N, real>::CTAS)
-    acoustic_tile_kernel(const StageParams<real> P, const uint32_t* __restrict__ face_tables) {
+    acoustic_tile_kernel(const LaneStageParams<real> P, const uint32_t* __restrict__ face_tables) {
   using C = TileCfg<N, real>;
   using R = FieldRhs<N, real>;
   using Tile = WarpTile<np3(N), real>;
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(128, TileCfg<N, real>::CTAS)
 // Projection and RK update of p from the bracket in P.rhs (kBracket): one warp
 // per 32 elements, blockDim.x / 32 warps per CTA (lane_launch).
 template <int N, int M, typename real>
-__global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS) acoustic_project_kernel(const StageParams<real> P) {
+__global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS) acoustic_project_kernel(const LaneStageParams<real> P) {
   using C = ProjectShape<N, M, real>;
   using Tile = WarpTile<np3(N), real>;
   using Pr = Projector<N, M, real, true>;
@@ -364,10 +364,10 @@ __global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS) acoustic_pr
       [&](int gl) { return P.steps_group && step_now >= P.steps_group[e0 + gl]; });
 }
 
-// The adjoint stage's update before its spatial operator (AdjPreParams), one
+// The adjoint stage's update before its spatial operator (LaneAdjPreParams), one
 // warp per 32 elements and field (blockIdx.x % 4).
 template <int N, int M, typename real>
-__global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS) lane_adj_pre_kernel(const AdjPreParams<real> P) {
+__global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS) lane_adj_pre_kernel(const LaneAdjPreParams<real> P) {
   using C = ProjectShape<N, M, real>;
   using Tile = WarpTile<np3(N), real>;
   using Pr = Projector<N, M, real, true>;
