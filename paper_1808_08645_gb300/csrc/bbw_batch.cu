@@ -366,12 +366,10 @@ bbw_status bbw_batch_create(int n, const int64_t* nverts, const double* const* v
     k.members = ids;
     int team = 0, V = 1, gpc = 1;
     bbw::ops_for(deg)->launch_shape(M, precision == 64, &team, &V, &gpc);
-    // the bucket's kernels go by its size (they give the same bits as a solo
-    // solver's); V = 1 with the tile kernels. Group padding only adds elements.
-    int64_t total = 0;
-    for (int i : ids) total += K[i];
-    if (bbw::ops_for(deg)->use_lane(M, precision == 64, total)) V = 1;
-    // disjoint union, every instance starting on a group boundary
+    // disjoint union, every instance starting on a group boundary of the team
+    // kernels. The solver below chooses its kernels by the union's size (they
+    // give the same bits as a solo solver's); with the tile kernels a padding
+    // element is a group of no instance, and the numbering stays the same.
     std::vector<double> xyz;
     std::vector<int64_t> tets;
     int64_t e = 0;
@@ -631,7 +629,7 @@ bbw_status bbw_batch_set_instance_steps(bbw_batch* b, const double* dt, const in
     if (k.d_stepsg) cudaFree(k.d_stepsg);
     k.d_dtg = nullptr;
     k.d_stepsg = nullptr;
-    // groups of no member (none exist: members tile the bucket) stay inert: dt 0, budget 0
+    // groups of no member (padding elements under the tile kernels) stay inert: dt 0, budget 0
     std::vector<double> gdt(size_t(s->G), 0.0);
     std::vector<int64_t> gst(size_t(s->G), 0);
     for (int i : k.members) {
