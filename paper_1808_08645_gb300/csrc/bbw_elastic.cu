@@ -31,7 +31,7 @@ struct bbw_elastic {
   void* d_geom = nullptr;   // [G][9][V]
   int32_t* d_conn = nullptr;  // [G][4][V]
   void* d_flux = nullptr;   // scratch of the kernels with one element per lane: face fluxes,
-  void* d_rhs = nullptr;    // brackets [K][10][Np]
+  void* d_trace = nullptr;  // stress trace [K][Np]
   double cs[bbw::kMaxN + 1] = {};  // constants of their projections
   void* d_stage = nullptr;  // FP64 user-layout staging of host state transfers
   std::vector<double> media;  // [3][K][Mp], caller's element order
@@ -87,10 +87,18 @@ int sm_count() {
 
 int conv_blocks(size_t n) { return int(std::min<size_t>((n + 255) / 256, size_t(sm_count()) * 16)); }
 
+// every array of the solver back to NULL
+void free_arrays(bbw_elastic* s) {
+  for (void** p : {&s->q[0], &s->q[1], &s->res, &s->d_media, &s->d_geom, reinterpret_cast<void**>(&s->d_conn),
+                   &s->d_flux, &s->d_trace, &s->d_stage}) {
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+  }
+}
+
 void free_elastic(bbw_elastic* s) {
   if (!s) return;
-  for (void* p : {s->q[0], s->q[1], s->res, s->d_media, s->d_geom, static_cast<void*>(s->d_conn), s->d_flux, s->d_rhs, s->d_stage})
-    if (p) cudaFree(p);
+  free_arrays(s);
   if (s->m) bbw_destroy(s->m);
   delete s;
 }
@@ -118,18 +126,13 @@ bbw_status upload_mesh(bbw_elastic* s) {
     const std::vector<real> rows = bbw::lane_geometry_rows<real>(m);
     BBW_CUDA(cudaMemcpy(s->d_geom, rows.data(), rows.size() * sizeof(real), cudaMemcpyHostToDevice));
   } else {
-  // geometry [G][9][V]: d lambda_m / d x for m = 1..3; padding: the unit tetrahedron
-  std::vector<double> g9(size_t(m->K) * 9);
-  for (int64_t e = 0; e < m->K; ++e)
-    for (int c = 0; c < 9; ++c) g9[size_t(e) * 9 + c] = m->grad[size_t(e) * 12 + 3 + c];
-  {
+    // geometry [G][9][V]: d lambda_m / d x for m = 1..3; padding: the unit tetrahedron
     std::vector<real> h(size_t(s->G) * 9 * V);
     for (int64_t e = 0; e < s->G * V; ++e)
       for (int c = 0; c < 9; ++c)
         h[(size_t(e / V) * 9 + c) * V + size_t(e % V)] =
-            real(e < m->K ? g9[size_t(m->user(e)) * 9 + c] : (c % 4 == 0 ? 1.0 : 0.0));
+            real(e < m->K ? m->grad[size_t(m->user(e)) * 12 + 3 + c] : (c % 4 == 0 ? 1.0 : 0.0));
     BBW_CUDA(cudaMemcpy(s->d_geom, h.data(), h.size() * sizeof(real), cudaMemcpyHostToDevice));
-  }
   }
   // connectivity [G][4][V]: (internal neighbour slot << 5) | (its face << 3) | orientation; -1: wall
   std::vector<int32_t> conn(size_t(s->G) * 4 * V, -1);
@@ -163,7 +166,7 @@ bbw_status launch(bbw_elastic* s, int stage, double dt) {
   P.tau_s = real(s->tau_s);
   P.status = m->d_status;
   P.flux = static_cast<real*>(s->d_flux);
-  P.rhs = static_cast<real*>(s->d_rhs);
+  P.trace = static_cast<real*>(s->d_trace);
   for (int j = 0; j <= m->N; ++j) P.cs[j] = real(s->cs[j]);
   BBW_CUDA(s->ops->launch(m->M, m->prec == 64, &P, s->grid, m->stream));
   s->cur = 1 - s->cur;
@@ -238,32 +241,41 @@ bbw_status bbw_elastic_create(int64_t nverts, const double* vxyz, int64_t K, con
     *p = nullptr;
   }
   s->ops = bbw::elastic_ops_for(N);
-  int team = 0, gpc = 1, per_sm = 0;
-  int width = 1;
-  size_t nflux = 0, nrhs = 0;
+  int team = 0, width = 1, gpc = 1, per_sm = 0;
+  size_t nflux = 0, ntrace = 0;
   s->ops->shape(M, precision == 64, &team, &width, &gpc);
-  s->V = s->ops->layout(M, precision == 64, K, &nflux, &nrhs);
+  s->V = s->ops->layout(M, precision == 64, K, &nflux, &ntrace);
   cudaError_t err = s->ops->prepare(M, precision == 64, &per_sm);
   if (err != cudaSuccess) {
     free_elastic(s);
     return fail(BBW_ERR_CUDA, std::string("elastic kernel set-up: ") + cudaGetErrorString(err));
   }
-  s->G = (K + s->V - 1) / s->V;
-  const int64_t tiles = (s->G + gpc - 1) / gpc;
-  s->grid = int(std::min<int64_t>(tiles, int64_t(std::max(1, per_sm)) * sm_count()));
   double c[5];
   bbw_lsrk_coeffs(s->rk_a, s->rk_b, c);
   s->ops->projection_scale(M, m->cj, s->cs);
   const size_t rs = s->rsz();
-  const size_t ng = size_t(s->G) * s->V;
   auto alloc = [&](void** p, size_t bytes) {
     return cudaMalloc(p, bytes) == cudaSuccess && cudaMemset(*p, 0, bytes) == cudaSuccess;
   };
-  const bool ok = alloc(&s->q[0], s->ninternal() * rs) && alloc(&s->q[1], s->ninternal() * rs) &&
-                  alloc(&s->res, s->ninternal() * rs) && alloc(&s->d_media, ng * 3 * m->Mp * rs) &&
-                  alloc(&s->d_geom, (nflux ? bbw::lane_geometry_values(K) : ng * 9) * rs) && alloc(reinterpret_cast<void**>(&s->d_conn), ng * 16) &&
-                  alloc(&s->d_stage, s->nuser() * 8) &&
-                  (!nflux || alloc(&s->d_flux, nflux * rs)) && (!nrhs || alloc(&s->d_rhs, nrhs * rs));
+  auto allocate = [&] {
+    s->G = (K + s->V - 1) / s->V;
+    const int64_t tiles = (s->G + gpc - 1) / gpc;
+    s->grid = int(std::min<int64_t>(tiles, int64_t(std::max(1, per_sm)) * sm_count()));
+    const size_t ng = size_t(s->G) * s->V;
+    return alloc(&s->q[0], s->ninternal() * rs) && alloc(&s->q[1], s->ninternal() * rs) &&
+           alloc(&s->res, s->ninternal() * rs) && alloc(&s->d_media, ng * 3 * m->Mp * rs) &&
+           alloc(&s->d_geom, (nflux ? bbw::lane_geometry_values(K) : ng * 9) * rs) &&
+           alloc(reinterpret_cast<void**>(&s->d_conn), ng * 16) && alloc(&s->d_stage, s->nuser() * 8) &&
+           (!nflux || (alloc(&s->d_flux, nflux * rs) && alloc(&s->d_trace, ntrace * rs)));
+  };
+  bool ok = allocate();
+  if (!ok && nflux) {  // the team kernel needs no scratch: it runs what the lane kernels' doesn't fit
+    cudaGetLastError();
+    free_arrays(s);
+    s->V = width;
+    nflux = ntrace = 0;
+    ok = allocate();
+  }
   if (!ok) {
     std::string msg = std::string("device allocation failed: ") + cudaGetErrorString(cudaGetLastError());
     free_elastic(s);

@@ -56,12 +56,9 @@ struct ElasticParams {
 // one struct, 39 without).
 template <typename real>
 struct LaneElasticParams : ElasticParams<real> {
-  // the fluxes at the face nodes [ceil(G / 32)][6][4][Nfp][32]; the brackets of
-  // the ten field tasks as power coefficients [G][10][Np] (fused kernels use
-  // the tenth alone, for the projected trace); the constants of the projection
-  real* __restrict__ flux = nullptr;
-  real* __restrict__ rhs = nullptr;
-  real cs[kMaxN + 1] = {};
+  real* __restrict__ flux = nullptr;   // at the face nodes [ceil(G / 32)][6][4][Nfp][32]
+  real* __restrict__ trace = nullptr;  // bracket of the stress trace, then its projection [G][Np]
+  real cs[kMaxN + 1] = {};             // constants of the projection
 };
 static_assert(offsetof(ElasticParams<float>, status) + sizeof(void*) == sizeof(ElasticParams<float>),
               "the team kernel's parameters hold nothing of the lane kernels'");

@@ -118,13 +118,13 @@ cudaError_t elaunch(int M, bool dbl, const void* params, int grid, cudaStream_t 
 }
 
 // Elements per group and scratch of a solver of K elements; see ElasticOps.
-int elayout(int M, bool dbl, int64_t K, size_t* flux, size_t* rhs) {
+int elayout(int M, bool dbl, int64_t K, size_t* flux, size_t* trace) {
   return edispatch(M, dbl, [&]<int MM, typename real>() {
-    *flux = *rhs = 0;
+    *flux = *trace = 0;
     if constexpr (kELane<real>) {
       if (K >= kELaneMin) {
         *flux = flux_values<6>(K, np2(kN));
-        *rhs = size_t(10) * size_t(K) * np3(kN);
+        *trace = size_t(K) * np3(kN);
         return 1;
       }
     }

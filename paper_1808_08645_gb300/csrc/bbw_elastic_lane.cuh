@@ -6,9 +6,14 @@
 // face of the field's flux (F_v,c, or A_n h combined from the three h before
 // the lift, since A_n is constant on an affine face), projection, RK update.
 // The trace of the stress bracket is a tenth task (div v and n . h), projected
-// with lambda ahead of the normal stresses, which add it to their own
-// projection with 2 mu. Ten independent tasks per 32 elements give every
-// degree enough warps, and no bracket leaves the chip.
+// with lambda in an earlier launch than the normal stresses, which add it to
+// their own projection with 2 mu. Ten tasks per 32 elements give every degree
+// enough warps. Up to N = 5 a task projects its bracket in registers; above,
+// the brackets of the nine fields wait for the projection kernels in their
+// fields' places of q_out, which nothing reads before the RK update writes
+// them. So only the fluxes and the trace take memory of their own,
+// 24 N_fp + N_p values an element, beside a state of 45 N_p (three copies in
+// FP32 and the FP64 staging).
 #pragma once
 
 #include "bbw_elastic.cuh"
@@ -74,13 +79,13 @@ __device__ __forceinline__ void elastic_finish(const LaneElasticParams<real>& P,
                                                int task) {
   using Tile = WarpTile<np3(N), real>;
   constexpr int Np = np3(N);
-  real* tr = P.rhs + (size_t(e0) * 10 + 9) * Np;
+  real* tr = P.trace + size_t(e0) * Np;
   if (task == 9) {
-    Tile::template unstage<10 * Np, S>(cols, tr, lane, ne);
+    Tile::template unstage<Np, S>(cols, tr, lane, ne);
     return;
   }
   if (task >= 3 && task < 6) {  // the lane adds to the column entries that it reads again below
-    const real* p = tr + Tile::template first<10 * Np>(lane);
+    const real* p = tr + Tile::template first<Np>(lane);
     real* c = cols + Tile::template first<S>(lane);
     constexpr int U = Tile::IT < 16 ? Tile::IT : 16;
 #pragma unroll
@@ -88,7 +93,7 @@ __device__ __forceinline__ void elastic_finish(const LaneElasticParams<real>& P,
       typename Tile::Chunk t[U];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (Tile::has(lane, i0 + u, ne)) t[u] = Tile::load(p + Tile::template offset<10 * Np>(i0 + u));
+        if (Tile::has(lane, i0 + u, ne)) t[u] = Tile::load(p + Tile::template offset<Np>(i0 + u));
 #pragma unroll
       for (int u = 0; u < U; ++u)
         if (Tile::has(lane, i0 + u, ne))
@@ -103,8 +108,8 @@ __device__ __forceinline__ void elastic_finish(const LaneElasticParams<real>& P,
 __device__ __forceinline__ int elastic_weight(int task) { return task < 3 ? 0 : task == 9 ? 1 : 2; }
 
 // One warp per 32 elements and task. FUSED: the tasks of one
-// launch are TRACE ? {trace, v_x, v_y, v_z} : the six stresses. Otherwise all
-// ten brackets go to P.rhs for elastic_project_kernel.
+// launch are TRACE ? {trace, v_x, v_y, v_z} : the six stresses. Otherwise the
+// brackets go to q_out and P.trace for elastic_project_kernel.
 template <int N, int M, typename real, bool FUSED, bool TRACE>
 __global__ void __launch_bounds__(FieldShape<N, real>::THREADS, N == 5 ? 2 : kFieldCtas<N>)
     elastic_field_kernel(const LaneElasticParams<real> P) {
@@ -144,12 +149,16 @@ __global__ void __launch_bounds__(FieldShape<N, real>::THREADS, N == 5 ? 2 : kFi
   } else {
     put_column(cols + lane * S, r);
     __syncwarp();
-    Tile::template unstage<10 * Np, S>(cols, P.rhs + (size_t(e0) * 10 + task) * Np, lane, ne);
+    if (task == 9)
+      Tile::template unstage<Np, S>(cols, P.trace + size_t(e0) * Np, lane, ne);
+    else
+      Tile::template unstage<9 * Np, S>(cols, P.qout + (size_t(e0) * 9 + task) * Np, lane, ne);
   }
 }
 
-// Projections and RK updates from the brackets in P.rhs, tasks per launch as in
-// the fused elastic_field_kernel.
+// Projections and RK updates from the brackets in q_out and P.trace, tasks per
+// launch as in the fused elastic_field_kernel. A warp reads its whole bracket
+// before it writes the field there.
 template <int N, int M, typename real, bool TRACE>
 __global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS)
     elastic_project_kernel(const LaneElasticParams<real> P) {
@@ -174,8 +183,11 @@ __global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS)
   real wc[Mp];
   const bool normal = !TRACE && task < 6;
   lane_weight<M, S>(wt, cols, lane, ne, normal ? real(2) : real(1), wc);
-  Tile::template stage<10 * Np, S, (Tile::IT < 28 ? Tile::IT : 28)>(cols, P.rhs + (size_t(e0) * 10 + task) * Np, lane,
-                                                                    ne);
+  constexpr int U = Tile::IT < 28 ? Tile::IT : 28;
+  if (task == 9)
+    Tile::template stage<Np, S, U>(cols, P.trace + size_t(e0) * Np, lane, ne);
+  else
+    Tile::template stage<9 * Np, S, U>(cols, P.qout + (size_t(e0) * 9 + task) * Np, lane, ne);
   __syncwarp();
   Projector<N, M, real>::run(cols + lane * S, cols + lane * S, cols + lane * S, wc, P.cs);
   __syncwarp();

@@ -19,8 +19,8 @@ struct ElasticOps {
   // launch shape: lanes per group, elements per group, groups per CTA
   void (*shape)(int M, bool dbl, int* team, int* group_width, int* groups_per_cta);
   // elements per group of the layout of a solver of K elements, and its scratch
-  // in values: face fluxes and brackets (0: the team kernel, which uses none)
-  int (*layout)(int M, bool dbl, int64_t K, size_t* flux, size_t* rhs);
+  // in values: face fluxes and the trace (0: the team kernel, which uses none)
+  int (*layout)(int M, bool dbl, int64_t K, size_t* flux, size_t* trace);
   // constants cs[N + 1] of the projection kernels from the N + 1 constants c_j
   void (*projection_scale)(int M, const double* cj, double* cs);
 };
