@@ -274,7 +274,7 @@ void free_solver(bbw_solver* s) {
   bbw::free_adjoint(s);
   for (void* p : {s->q[0], s->q[1], s->res, s->d_c2, s->d_geom, static_cast<void*>(s->d_conn), s->d_src,
                   static_cast<void*>(s->d_src_groups), static_cast<void*>(s->d_src_slots),
-                  static_cast<void*>(s->d_src_ser), static_cast<void*>(s->d_src_amp), s->d_stage, s->d_rhs,
+                  static_cast<void*>(s->d_src_ser), static_cast<void*>(s->d_src_amp), s->d_stage,
                   static_cast<void*>(s->d_perm),
                   static_cast<void*>(s->d_inv),
                   static_cast<void*>(s->d_status)})
@@ -786,8 +786,6 @@ bbw_status bbw::create_solver(int64_t nverts, const double* vxyz, int64_t K, con
             alloc(&s->res, s->nstate_internal() * rs) && alloc(&s->d_c2, ng * s->Mp * rs) &&
             alloc(&s->d_geom, ng * 9 * rs) && alloc(reinterpret_cast<void**>(&s->d_conn), ng * 16) &&
             alloc(reinterpret_cast<void**>(&s->d_status), 16);
-  const size_t nrhs = s->lane ? s->ops->lane_scratch(precision == 64, K) : 0;
-  ok = ok && (!nrhs || alloc(&s->d_rhs, nrhs * rs));
   if (!ok) {
     std::string msg = std::string("device allocation failed: ") + cudaGetErrorString(cudaGetLastError());
     free_solver(s);

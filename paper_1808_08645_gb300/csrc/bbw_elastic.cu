@@ -236,7 +236,7 @@ bbw_status bbw_elastic_create(int64_t nverts, const double* vxyz, int64_t K, con
   }
   bbw_solver* m = s->m;
   // the acoustic state, c^2 and layout buffers are not used
-  for (void** p : {&m->q[0], &m->q[1], &m->res, &m->d_c2, &m->d_geom, reinterpret_cast<void**>(&m->d_conn), &m->d_rhs}) {
+  for (void** p : {&m->q[0], &m->q[1], &m->res, &m->d_c2, &m->d_geom, reinterpret_cast<void**>(&m->d_conn)}) {
     if (*p) cudaFree(*p);
     *p = nullptr;
   }

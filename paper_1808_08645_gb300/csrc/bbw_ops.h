@@ -34,8 +34,6 @@ struct KernelOps {
   // whether a solver of K elements runs the tile kernels (bbw_tile.cuh; the
   // launch entries do so when the parameters' lane is set)
   bool (*use_lane)(int M, bool dbl, int64_t K);
-  // values of their p bracket buffer for K elements (0: not used)
-  size_t (*lane_scratch)(bool dbl, int64_t K);
 };
 
 const KernelOps& ops_n1();

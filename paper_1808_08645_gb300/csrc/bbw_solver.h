@@ -77,7 +77,6 @@ struct bbw_solver {
   void* pinned = nullptr;
   size_t pinned_bytes = 0;
   bool lane = false;        // the tile kernels (one element per lane): V = 1
-  void* d_rhs = nullptr;    // their p bracket [K][Np]
   void* d_stage = nullptr;  // FP64 user-layout staging of host state transfers
   size_t d_stage_bytes = 0;
   int cur = 0;
@@ -158,11 +157,10 @@ void set_stage_sources(const bbw_solver* s, P_t& P, int64_t step, int stage, boo
   P.stage = stage;
 }
 
-// Which kernels a launch of solver s runs, and their scratch and constants.
+// Which kernels a launch of solver s runs, and their constants.
 template <typename P_t, typename real>
 void set_lane(const bbw_solver* s, P_t& P) {
   P.lane = s->lane;
-  P.rhs = static_cast<real*>(s->d_rhs);
   for (int j = 0; j <= s->N; ++j) P.cs[j] = real(s->cj[j]);
 }
 

@@ -101,8 +101,7 @@ struct StageParams {
 template <typename real>
 struct LaneStageParams : StageParams<real> {
   bool lane = false;
-  real* __restrict__ rhs = nullptr;  // p bracket between the tile and the projection kernel [G][Np]
-  real cs[kMaxN + 1] = {};           // the c_j
+  real cs[kMaxN + 1] = {};  // the c_j
 };
 
 // One stage of the discrete adjoint before its spatial operator, in the

@@ -238,10 +238,6 @@ bool use_lane(int M, bool dbl, int64_t K) {
   return dispatch(M, dbl, [&]<int MM, typename real>() { return kLane<real> && K >= kLaneMin<real>; });
 }
 
-size_t lane_scratch(bool dbl, int64_t K) {
-  return (dbl ? kFuseProjection<double> : kFuseProjection<float>) ? 0 : size_t(K) * np3(kN);
-}
-
 }  // namespace
 
 #define BBW_CAT2(a, b) a##b
@@ -249,7 +245,7 @@ size_t lane_scratch(bool dbl, int64_t K) {
 const KernelOps& BBW_CAT(ops_n, BBW_N)() {
   static const KernelOps ops = {&tables_size,  &build,          &face_maps,    &prepare,
                                 &launch_stage, &launch_wadg,    &launch_shape, &launch_spatial,
-                                &check_tables, &launch_adj_pre, &use_lane,     &lane_scratch};
+                                &check_tables, &launch_adj_pre, &use_lane};
   return ops;
 }
 

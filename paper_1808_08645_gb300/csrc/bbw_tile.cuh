@@ -33,7 +33,8 @@
 
 namespace bbw {
 
-// kBracket: the p bracket goes to P.rhs for acoustic_project_kernel;
+// kBracket: the p bracket goes to p's place in q_out, which nothing reads before
+// the RK update writes it, for acoustic_project_kernel;
 // kSpatial: the spatial operator alone (as the SP form of stage_kernel).
 enum TileMode { kFused = 0, kBracket = 1, kSpatial = 2 };
 
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(128, TileCfg<N, real>::CTAS)
       } else {
         put_column(col, r);
         __syncwarp();
-        Tile::template unstage<Np, S>(cols, P.rhs + size_t(e0) * Np, lane, ne);
+        Tile::template unstage<ES, S>(cols, P.qout + base, lane, ne);
       }
     }
     if (MODE == kFused || fld != 0) {
@@ -353,8 +354,9 @@ __global__ void __launch_bounds__(128, TileCfg<N, real>::CTAS)
   }
 }
 
-// Projection and RK update of p from the bracket in P.rhs (kBracket): one warp
-// per 32 elements, blockDim.x / 32 warps per CTA (lane_launch).
+// Projection and RK update of p from the bracket in q_out (kBracket), which the
+// warp reads whole before it writes p there: one warp per 32 elements,
+// blockDim.x / 32 warps per CTA.
 template <int N, int M, typename real>
 __global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS) acoustic_project_kernel(const LaneStageParams<real> P) {
   using C = ProjectShape<N, M, real>;
@@ -375,7 +377,7 @@ __global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS) acoustic_pr
   if (P.a != real(0)) Tile::template prefetch<4 * Np>(P.res + size_t(e0) * 4 * Np, lane, ne);
   real wc[Mp];
   lane_weight<M, S>(wt, cols, lane, ne, real(1), wc);
-  Tile::template stage<Np, S, (Tile::IT < 28 ? Tile::IT : 28)>(cols, P.rhs + size_t(e0) * Np, lane, ne);
+  Tile::template stage<4 * Np, S, (Tile::IT < 28 ? Tile::IT : 28)>(cols, P.qout + size_t(e0) * 4 * Np, lane, ne);
   __syncwarp();
   real* col = cols + lane * S;
   if constexpr (N > Pr::RD) {
