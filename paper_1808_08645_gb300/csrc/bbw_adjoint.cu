@@ -91,6 +91,7 @@ struct AdjointData {
   void* d_invf = nullptr;
   void* d_gw = nullptr;
   int ngam = 0;
+  int row = 32;  // stride of the gradient kernel's staged operands (grad_shape)
   int32_t* d_split = nullptr;  // gamma ranges of the gradient kernel's warps [kGradWarps + 1]
   bool grad_ready = false;  // the gradient kernel's shared-memory attribute is set
   int nsm = 0;              // SMs of the device
@@ -145,7 +146,7 @@ __global__ void receiver_adjoint_kernel(real* __restrict__ kap, const int64_t* _
 
 // gc[e][b] += dt sum_gamma G[gamma][b] sum_{(a, a') in pairs(gamma)} rho_p[e][a] / a! * v[e][a'] / a'!.
 // A block of kGradWarps warps takes 32 consecutive (internal) elements, one
-// per lane. The operands are staged once per block as [Np][32] columns; warp
+// per lane. The operands are staged once per block as [Np][row] columns; warp
 // q walks the gamma range [split.c[q], split.c[q + 1]) (ranges balanced by
 // pair count on the host), all its lanes in step over the same pair list, so
 // table words are broadcast loads and each lane reads only its own column
@@ -153,14 +154,14 @@ __global__ void receiver_adjoint_kernel(real* __restrict__ kap, const int64_t* _
 // holds the ranges (device memory). The warps' partial sums
 // are added in warp order (deterministic). rho_p is field 0 of the internal
 // [G][4][Np][V] layout, v the pressure bracket [G][Np][V]. Pair words hold
-// (32 a) | (32 a') << 16, the operand offsets in the columns. With SMEM the
+// (row a) | (row a') << 16, the operand offsets in the columns. With SMEM the
 // tables (G, pairs, row pointers; tab_bytes) are first copied into shared
 // memory, otherwise read from global memory (uniform loads).
 template <typename real, bool SMEM>
 __global__ void __launch_bounds__(32 * kGradWarps) adj_grad_kernel(
     const real* __restrict__ rho, const real* __restrict__ v, real* __restrict__ gc, int64_t K, int Np, int Mp, int V,
     int ngam, const int32_t* __restrict__ gptr_g, const uint32_t* __restrict__ pairs_g, const real* __restrict__ invf,
-    const real* __restrict__ gw_g, real dt, int tab_bytes, const int32_t* __restrict__ split) {
+    const real* __restrict__ gw_g, real dt, int tab_bytes, const int32_t* __restrict__ split, int row) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int32_t* gptr = gptr_g;
@@ -178,21 +179,41 @@ __global__ void __launch_bounds__(32 * kGradWarps) adj_grad_kernel(
     gw = gws;
   }
   real* rs0 = reinterpret_cast<real*>(sm_raw + tab_bytes);
-  real* vs0 = rs0 + size_t(Np) * 32;
-  real* part = vs0 + size_t(Np) * 32;  // [kGradWarps][Mp][32]
+  real* vs0 = rs0 + size_t(Np) * row;
+  real* part = vs0 + size_t(Np) * row;  // [kGradWarps][Mp][32]
   const real* rs = rs0 + lane;
   const real* vs = vs0 + lane;
   const int c_lo = split[w], c_hi = split[w + 1];
   for (int64_t e0 = int64_t(blockIdx.x) * 32; e0 < K; e0 += int64_t(gridDim.x) * 32) {
-    {  // stage the 32 elements' operands, warp w taking rows w, w + 8, ...
+    if (row == 33) {
+      // V = 1: the warp takes whole runs of an element's coefficients (lanes on
+      // elements would read 32 sectors for 32 values: N = 5,
+      // 24,576 elements, 83.3 us a launch, with runs 71.3)
+      constexpr int EW = 32 / kGradWarps;  // elements per warp, all in flight
+      for (int i = lane; i < Np; i += 32) {
+        const real f = invf[i];
+        real r[EW], u[EW];
+#pragma unroll
+        for (int x = 0; x < EW; ++x) {
+          const int64_t e = e0 + w * EW + x;
+          r[x] = e < K ? rho[size_t(e) * 4 * Np + i] : real(0);
+          u[x] = e < K ? v[size_t(e) * Np + i] : real(0);
+        }
+#pragma unroll
+        for (int x = 0; x < EW; ++x) {
+          rs0[i * row + w * EW + x] = r[x] * f;
+          vs0[i * row + w * EW + x] = u[x] * f;
+        }
+      }
+    } else {  // warp w takes rows w, w + 8, ... of the groups
       const int64_t e = e0 + lane;
       const bool ok = e < K;
       const int64_t g = ok ? e / V : 0;
       const int l = ok ? int(e % V) : 0;
       for (int i = w; i < Np; i += kGradWarps) {
         const real f = invf[i];
-        rs0[i * 32 + lane] = ok ? rho[(size_t(g) * 4 * Np + i) * V + l] * f : real(0);
-        vs0[i * 32 + lane] = ok ? v[(size_t(g) * Np + i) * V + l] * f : real(0);
+        rs0[i * row + lane] = ok ? rho[(size_t(g) * 4 * Np + i) * V + l] * f : real(0);
+        vs0[i * row + lane] = ok ? v[(size_t(g) * Np + i) * V + l] * f : real(0);
       }
     }
     __syncthreads();
@@ -242,6 +263,25 @@ bbw_status upload_real(const std::vector<double>& h, void** d) {
   return BBW_OK;
 }
 
+// Shared memory of the gradient kernel with operand rows of `row` values:
+// tables where they fit beside the staged operands and the partial sums, and
+// as many blocks per SM as that leaves (at most 8).
+struct GradShape {
+  size_t tab, bytes;
+  bool in_smem;
+  int per_sm;
+};
+GradShape grad_shape(const bbw_solver* s, int ngam, int row, size_t rs) {
+  GradShape g;
+  const size_t cap = size_t(bbw::kSmemPerCta);
+  const size_t ops = (size_t(2) * s->Np * row + size_t(kGradWarps) * s->Mp * 32) * rs;
+  g.tab = (size_t(ngam) * s->Mp * rs + size_t(s->Np) * s->Np * 4 + size_t(ngam + 1) * 4 + 15) / 16 * 16;
+  g.in_smem = g.tab + ops <= cap;
+  g.bytes = (g.in_smem ? g.tab : 0) + ops;
+  g.per_sm = int(std::max<size_t>(1, std::min<size_t>(8, cap / g.bytes)));
+  return g;
+}
+
 // The gradient tables of the degree-2N product (see the file comment).
 template <typename real>
 bbw_status build_tables(bbw_solver* s, AdjointData* a) {
@@ -255,13 +295,16 @@ bbw_status build_tables(bbw_solver* s, AdjointData* a) {
     return bbw::idx3(2 * N, g[1], g[2], g[3]);
   };
   const int ngam = int(G2.size());
+  // with V = 1 the staging transposes, which takes an odd row where that costs
+  // no resident block (it does at N = 9, M = 0 in FP64, and at N = M = 2 there)
+  a->row = s->V == 1 && grad_shape(s, ngam, 33, sizeof(real)).per_sm == grad_shape(s, ngam, 32, sizeof(real)).per_sm ? 33 : 32;
   std::vector<std::vector<uint32_t>> by(static_cast<size_t>(ngam));
   for (int i = 0; i < Np; ++i)
     for (int j = 0; j < Np; ++j) {
       std::array<int, 4> g;
       for (int x = 0; x < 4; ++x) g[x] = A[size_t(i)][x] + A[size_t(j)][x];
-      // offsets of the two operands in the warp's staged [Np][32] columns
-      by[size_t(idx2n(g))].push_back(uint32_t(32 * i) | (uint32_t(32 * j) << 16));
+      // offsets of the two operands in the staged rows
+      by[size_t(idx2n(g))].push_back(uint32_t(a->row * i) | (uint32_t(a->row * j) << 16));
     }
   std::vector<int32_t> gptr(size_t(ngam) + 1, 0);
   std::vector<uint32_t> pairs;
@@ -399,12 +442,8 @@ bbw_status adjoint_stage(bbw_solver* s, AdjointData* a, const void* vbr, int sta
   bbw::set_stage_sources<bbw::LaneStageParams<real>, real>(s, P, 0, stage, false);
   BBW_CUDA(s->ops->launch_spatial(s->M, s->prec == 64, &P, s->grid_stage, st));
   // gc += dt rho_t,p^T T_beta v
-  const size_t ops = (size_t(2) * s->Np + size_t(kGradWarps) * s->Mp) * 32 * sizeof(real);  // staged operands, partials
-  const size_t tab = (size_t(a->ngam) * s->Mp * sizeof(real) + size_t(s->Np) * s->Np * 4 + size_t(a->ngam + 1) * 4 +
-                      15) / 16 * 16;
-  const size_t cap = size_t(bbw::kSmemPerCta);
-  const bool in_smem = tab + ops <= cap;
-  const size_t bytes = (in_smem ? tab : 0) + ops;
+  const GradShape gs = grad_shape(s, a->ngam, a->row, sizeof(real));
+  const size_t bytes = gs.bytes, cap = size_t(bbw::kSmemPerCta);
   if (bytes > cap) return fail(BBW_ERR_ARG, "adjoint gradient: staged operands exceed shared memory");
   if (!a->grad_ready) {
     BBW_CUDA(cudaFuncSetAttribute(adj_grad_kernel<real, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -416,16 +455,14 @@ bbw_status adjoint_stage(bbw_solver* s, AdjointData* a, const void* vbr, int sta
     BBW_CUDA(cudaDeviceGetAttribute(&a->nsm, cudaDevAttrMultiProcessorCount, dev));
     a->grad_ready = true;
   }
-  // blocks per SM: as many as the shared memory holds (at most 8)
-  const int per_sm = int(std::max<size_t>(1, std::min<size_t>(8, cap / bytes)));
-  const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((s->K + 31) / 32, int64_t(std::max(a->nsm, 1)) * per_sm)));
+  const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((s->K + 31) / 32, int64_t(std::max(a->nsm, 1)) * gs.per_sm)));
   auto launch = [&](auto kern) {
     kern<<<blocks, 32 * kGradWarps, bytes, st>>>(
         static_cast<const real*>(a->rho), static_cast<const real*>(vbr), static_cast<real*>(a->gc), s->K, s->Np, s->Mp,
         s->V, a->ngam, a->d_gptr, a->d_pairs, static_cast<const real*>(a->d_invf), static_cast<const real*>(a->d_gw),
-        real(dt), in_smem ? int(tab) : 0, a->d_split);
+        real(dt), gs.in_smem ? int(gs.tab) : 0, a->d_split, a->row);
   };
-  if (in_smem)
+  if (gs.in_smem)
     launch(adj_grad_kernel<real, true>);
   else
     launch(adj_grad_kernel<real, false>);
