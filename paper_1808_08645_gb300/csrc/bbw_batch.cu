@@ -706,7 +706,9 @@ bbw_status bbw_batch_autotune(bbw_batch* b, int steps, int* schedule, double* ms
     bool serial;
     double factor;
   } cand[] = {{false, 1.0}, {true, 1.0}, {false, 0.5}, {false, 2.0}};
-  constexpr int ncand = int(sizeof(cand) / sizeof(cand[0]));
+  // (the grid goes to the team kernels alone: without one there are no grids to try)
+  const bool tiles_only = std::all_of(b->buckets.begin(), b->buckets.end(), [](const auto& k) { return k.s->lane; });
+  const int ncand = tiles_only ? 2 : int(sizeof(cand) / sizeof(cand[0]));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   BBW_CUDA(cudaEventCreate(&e0));
   BBW_CUDA(cudaEventCreate(&e1));

@@ -214,3 +214,10 @@ def test_per_instance_dt_and_step_budgets_match_solo_runs(prec, graph):
     with pytest.raises(B.BBWError):
         b.set_instance_steps(None, np.full(n, -1))
     b.close()
+
+
+def test_autotune_tries_no_grids_where_they_have_no_effect():
+    """The grid factors (schedules 2 and 3) scale the team kernels' persistent grids. N = 5 runs the tile kernels at every
+    size, which take one CTA per tile: only the order of the buckets is tried."""
+    with B.Batch([inputs.cube_mesh(3), inputs.cube_mesh(4)], [5, 5], 2, 32) as b:
+        assert all(b.autotune(1)[0] <= 1 for _ in range(12))
