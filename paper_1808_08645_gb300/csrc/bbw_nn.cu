@@ -320,8 +320,9 @@ __global__ void __launch_bounds__(THREADS, 4) gemm_bf16_kernel(const float* __re
 // thread take two pencils instead of four and twice the threads hide the
 // latency of the field (a training step on the 64^3 grid, 6 modes: 7.04 ms
 // before, 6.14 with). Bases whose padded rows exceed the 48 KB of shared
-// memory that need no opt-in, and more than 8 modes, where two pencils fill
-// the registers already, read unpadded rows.
+// memory that need no opt-in, more than 8 modes, where two pencils fill the
+// registers already, and the sums that bbw_nn_axis_transform names, read
+// unpadded rows.
 constexpr int kMaxModes = 16;
 template <int MM>
 struct BasisRow {
@@ -615,7 +616,17 @@ bbw_status bbw_nn_axis_transform(const float* basis, int L, int m, const float* 
                                                                    act);
   };
   const size_t shm = size_t(L) * m * sizeof(float);
-  if (m <= 8 && size_t(L) * 8 * sizeof(float) <= 48 * 1024)
+  // A sum over z (expand = 0) takes a thread as long with four pencils as 1.2
+  // to 1.35 times two, so four are the better choice where they halve the blocks
+  // on the fullest SM, from two to one or, while the field stays in L2, from four
+  // to two: L = 64, m = 6, C = 32, at 4,096 pencils 12.3 us with four and 14.4
+  // with two, at 8,192 20.5 and 25.4; at 2,400 (one block either way) 12.3 and
+  // 10.3, at 5,200 (two and three) 20.0 and 18.5. Expansions are faster with two
+  // at every size (4,096 pencils: 38.7 and 30.7).
+  auto per_sm = [&](int pp) { return ((pencils + pp - 1) / pp * C + 256 * 152 - 1) / (256 * 152); };
+  const bool four = !expand && per_sm(2) == 2 * per_sm(4) &&
+                    (per_sm(4) == 1 || (per_sm(4) == 2 && pencils * L * C * 4 <= (96LL << 20)));
+  if (m <= 8 && !four && size_t(L) * 8 * sizeof(float) <= 48 * 1024)
     launch(axis_transform_kernel<8, 2, true>, 2, size_t(L) * 8 * sizeof(float));
   else if (m <= 8)
     launch(axis_transform_kernel<8, 4, false>, 4, shm);
