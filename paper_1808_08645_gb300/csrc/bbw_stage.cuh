@@ -283,10 +283,41 @@ __device__ __forceinline__ vec<real, V> vaxpy(const vec<real, V>& a, real w, con
   vfmas(r, w, b);
   return r;
 }
+// Products and differences that are not contracted into an FMA. What the tile
+// kernels (bbw_tile.cuh) repeat bit by bit is written with these and with fma,
+// so that the rounding is the source's and not the compiler's choice.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+
+// |g|^2, in an order that goes with the width of the solver's group
+template <int V, typename real>
+__device__ __forceinline__ real norm2(real gx, real gy, real gz) {
+  return V == 2 ? fma(gz, gz, fma(gx, gx, mul_rn(gy, gy))) : fma(gz, gz, fma(gy, gy, mul_rn(gx, gx)));
+}
+
+// tau x - y: the product rounded on its own in FP32, as the packed products
+// are, and contracted in FP64
+__device__ __forceinline__ float penalty(float tau, float x, float y) { return sub_rn(mul_rn(tau, x), y); }
+__device__ __forceinline__ double penalty(double tau, double x, double y) { return fma(tau, x, -y); }
+
 // a - b
 template <typename real, int V>
 __device__ __forceinline__ vec<real, V> vsub(const vec<real, V>& a, const vec<real, V>& b) {
   return vaxpy(a, real(-1), b);
+}
+// penalty(tau, a, b)
+template <typename real, int V>
+__device__ __forceinline__ vec<real, V> vpenalty(real tau, const vec<real, V>& a, const vec<real, V>& b) {
+  if constexpr (sizeof(real) == 4 && V % 2 == 0) {
+    return vsub(vmuls(tau, a), b);
+  } else {
+    vec<real, V> r;
+#pragma unroll
+    for (int i = 0; i < V; ++i) r.x[i] = penalty(tau, a.x[i], b.x[i]);
+    return r;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -520,8 +551,12 @@ __device__ __forceinline__ void wadg_group(const Tables<N, M, real>& tab, real* 
         if (s.w1 > 0) vfmas(acc, real(s.w1), vld<real, V>(X + (s.base - 1) * V));
         if (s.w2 > 0) vfmas(acc, real(s.w2), vld<real, V>(X + (s.base - s.dk) * V));
         if (s.w3 > 0) vfmas(acc, real(s.w3), vld<real, V>(X + (s.base - s.dl) * V));
-        w[r] = vmuls(c, lv[jl][r]);
-        vfmas(w[r], inv, acc);
+        if (n == 1) {  // 1/n = 1: one FMA
+          w[r] = vaxpy(acc, c, lv[jl][r]);
+        } else {
+          w[r] = vmuls(c, lv[jl][r]);
+          vfmas(w[r], inv, acc);
+        }
       }
     }
     if (jl > 0) {
@@ -661,7 +696,7 @@ __global__ void __launch_bounds__(T* GC) stage_kernel(const StageParams<real> P)
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         const real gx = fx.get(v), gy = fy.get(v), gz = fz.get(v);
-        const real gn = sqrt(gx * gx + gy * gy + gz * gz);
+        const real gn = sqrt(norm2<V>(gx, gy, gz));
         const real inv = real(1) / gn;
         real* nr = NRM + 4 * t * V + v;
         nr[0] = -gx * inv;
@@ -785,8 +820,8 @@ __global__ void __launch_bounds__(T* GC) stage_kernel(const StageParams<real> P)
         vt ndu = vmul(nx, vsub(up, um));
         vfma(ndu, ny, vsub(vp, vm));
         vfma(ndu, nz, vsub(wp, wm));
-        vst(trace(0, f, a), vmul(hs, vaxpy(vmuls(P.tau_p, jp), real(-1), ndu)));
-        vst(trace(1, f, a), vmul(hs, vaxpy(vmuls(P.tau_u, ndu), real(-1), jp)));
+        vst(trace(0, f, a), vmul(hs, vpenalty(P.tau_p, jp, ndu)));
+        vst(trace(1, f, a), vmul(hs, vpenalty(P.tau_u, ndu, jp)));
       }
     }
     team_sync<T>();

@@ -42,17 +42,6 @@ enum TileMode { kFused = 0, kBracket = 1, kSpatial = 2 };
 // addition with the product that x is
 __device__ __forceinline__ void keep(float& x) { asm volatile("" : "+f"(x)); }
 __device__ __forceinline__ void keep(double& x) { asm volatile("" : "+d"(x)); }
-// products and differences that are not contracted into an FMA
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
-
-// tau x - y as stage_kernel computes it: packed FP32 rounds the product, FP64
-// is contracted
-__device__ __forceinline__ float penalty(float tau, float x, float y) { return sub_rn(mul_rn(tau, x), y); }
-__device__ __forceinline__ double penalty(double tau, double x, double y) { return fma(tau, x, -y); }
-
 template <int N, typename real>
 struct TileCfg {
   static constexpr int Np = np3(N), Nfp = np2(N), ITEMS = 4 * Nfp;
@@ -140,10 +129,7 @@ __global__ void __launch_bounds__(128, TileCfg<N, real>::CTAS)
       g[d] = f == 0 ? -g1 - g2 - g3 : f == 1 ? g1 : f == 2 ? g2 : g3;
     }
     const real gx = g[0], gy = g[1], gz = g[2];
-    // |g|^2 in the order that the compiler contracts it in stage_kernel, which
-    // goes with its group width
-    const real gn = TileShape<N, real>::V == 2 ? sqrt(fma(gz, gz, fma(gx, gx, mul_rn(gy, gy))))
-                                               : sqrt(fma(gz, gz, fma(gy, gy, mul_rn(gx, gx))));
+    const real gn = sqrt(norm2<TileShape<N, real>::V>(gx, gy, gz));
     const real inv = real(1) / gn;
     real* nr = NRM + f * 128 + e;
     nr[0] = -gx * inv;
