@@ -71,7 +71,7 @@ cudaError_t eprepare(int M, bool dbl, int* per_sm) {
     auto k = elastic_fn<MM, real>();
     cudaError_t err = allow(k, C::SMEM);
     if constexpr (kELane<real>) {
-      if (err == cudaSuccess) err = allow(elastic_flux_kernel<kN, real>, flux_smem<kN, 6, real>());
+      if (err == cudaSuccess) err = allow(elastic_flux_kernel<kN, real>, flux_smem<kN, real>());
       if (err == cudaSuccess) err = allow(efield_fn<MM, real, true>(), EFCfg<MM, real>::SMEM);
       if constexpr (kEFused) {
         if (err == cudaSuccess) err = allow(efield_fn<MM, real, false>(), EFCfg<MM, real>::SMEM);
@@ -94,7 +94,7 @@ cudaError_t elaunch(int M, bool dbl, const void* params, int grid, cudaStream_t 
         using Tab = Tables<kN, MM, real>;
         const char* t = static_cast<const char*>(P.tables);
         elastic_flux_kernel<kN, real>
-            <<<unsigned((P.G + kFluxTile<kN, 6> - 1) / kFluxTile<kN, 6>), kFluxThreads, flux_smem<kN, 6, real>(), s>>>(
+            <<<unsigned((P.G + kFluxTile<kN> - 1) / kFluxTile<kN>), kFluxThreads, flux_smem<kN, real>(), s>>>(
                 P, reinterpret_cast<const uint16_t*>(t + offsetof(Tab, fidx)),
                 reinterpret_cast<const uint16_t*>(t + offsetof(Tab, nidx)));
         auto blocks = [&](int warps) { return unsigned((P.G + 32 * warps - 1) / (32 * warps)); };
@@ -123,7 +123,7 @@ int elayout(int M, bool dbl, int64_t K, size_t* flux, size_t* trace) {
     *flux = *trace = 0;
     if constexpr (kELane<real>) {
       if (K >= kELaneMin) {
-        *flux = flux_values<6>(K, np2(kN));
+        *flux = flux_values(K, np2(kN));
         *trace = size_t(K) * np3(kN);
         return 1;
       }

@@ -1,27 +1,11 @@
 // bbw_lane.cuh -- the spatial operator and the RK update with one element per
 // lane: the parts shared by the acoustic tile kernel (bbw_tile.cuh) and the
-// elastic field tasks (bbw_elastic_lane.cuh), and the elastic form, two kinds
-// of kernels per stage:
-//   flux kernel   the penalty fluxes at the face nodes of every element, with
-//                 one face node per lane (neighbour traces are short runs of
-//                 the neighbour's field, so a warp's gather covers few
-//                 sectors), transposed through shared memory to [32 elements]
-//                 lines;
-//   field tasks   one warp per 32 elements and field, one element per lane:
-//                 derivative terms, lift of the four faces, the projection
-//                 (bbw_project.cuh) and the RK update.
+// elastic field tasks (bbw_elastic_lane.cuh).
 // A field's right-hand side is  E sum_t D_{d_t} f_t + sum_face L^f F: with the
 // element in a lane every stencil index and weight is an immediate, the degree
 // N-1 combination (V1), the lift pyramid and the right-hand side are registers
 // (N_p <= 120: up to N = 7), and shared memory only transposes between the
-// lanes' elements and contiguous global accesses. Nothing is shared between
-// warps, so they never wait for each other.
-//
-// The field tasks of the same elements run in neighbouring CTAs, so that their
-// common inputs come from L2 (task-major order took 1.8 times the DRAM bytes).
-// Registers bound the warps per SM (8 to 24); the code of a task (30 to 100 KB)
-// exceeds the instruction cache from N = 5 on, which is why warps of a CTA, in
-// step with each other, do better than as many smaller CTAs.
+// lanes' elements and contiguous global accesses.
 #pragma once
 
 #include "bbw_project.cuh"
@@ -29,158 +13,6 @@
 #include "bbw_warp_tile.cuh"
 
 namespace bbw {
-
-// Physics descriptions: fields, flux quantities and the terms of each field
-// task. Derivative term t adds sgn * d f / d x_d; lift term t the flux
-// quantity q times n_d (d < 0: times 1).
-struct Term {
-  int8_t what, dir;
-};
-struct TaskDesc {
-  int nd, nl;
-  Term d[3];
-  Term l[3];
-};
-
-// Flux kernel: 4 warps per CTA and a tile of 16 elements, 8 where 16 elements'
-// fluxes would take the shared memory that the gathers need as L1.
-constexpr int kFluxThreads = 128;
-template <int N, int NQ>
-constexpr int kFluxTile = NQ * 4 * np2(N) <= 224 ? 16 : 8;
-
-template <int N, int NQ, typename real>
-constexpr int flux_smem() {
-  // fluxes [NQ][4 Nfp][tile + 1] | normals [tile][4][4] | connectivity [tile][4]
-  constexpr int T = kFluxTile<N, NQ>;
-  return int(sizeof(real)) * (NQ * 4 * np2(N) * (T + 1) + T * 16) + T * 16;
-}
-// values of the flux buffer of K elements (whole tiles of 32)
-template <int NQ>
-constexpr size_t flux_values(int64_t K, int Nfp) {
-  return size_t((K + 31) / 32) * 32 * NQ * 4 * size_t(Nfp);
-}
-
-// The fluxes of a tile: flux(nrm, own[NF], nb[NF], out[NQ]) per face node.
-// Walls: mirror(own, nb). Layout of P.flux: [K / 32][NQ][4][Nfp][32].
-template <typename Phys, int N, typename real, typename Params, typename Mirror, typename Flux>
-__device__ __forceinline__ void flux_tile(const Params& P, const uint16_t* __restrict__ fidx,
-                                          const uint16_t* __restrict__ nidx, Mirror&& mirror, Flux&& flux) {
-  constexpr int Np = np3(N), Nfp = np2(N), NF = Phys::NF, NQ = Phys::NQ, ITEMS = 4 * Nfp;
-  constexpr int T = kFluxTile<N, NQ>, ST = T + 1;
-  extern __shared__ __align__(16) unsigned char smem[];
-  real* FL = reinterpret_cast<real*>(smem);           // [NQ][4 Nfp][ST]
-  real* NRM = FL + NQ * ITEMS * ST;                   // [tile][4][nx, ny, nz, |f| / (2 |D|)]
-  int* CS = reinterpret_cast<int*>(NRM + T * 16);  // [tile][4]
-  const int64_t e0 = int64_t(blockIdx.x) * T;
-  const int ne = P.G - e0 < T ? int(P.G - e0) : T;
-  const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
-  bool oob = false;
-  (void)oob;
-  if (tid < 4 * T) {
-    const int e = tid / 4, f = tid % 4;
-    if (e < ne) {
-      CS[tid] = P.conn[size_t(e0 + e) * 4 + f];
-      const real* g = P.geom + size_t((e0 + e) / 32) * 32 * kLaneGeom + (e0 + e) % 32;
-      const real inv = g[(9 + f) * 32];
-      real* nr = NRM + tid * 4;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const real a = g[d * 32], b = g[(3 + d) * 32], c = g[(6 + d) * 32];
-        nr[d] = (f == 0 ? a + b + c : f == 1 ? -a : f == 2 ? -b : -c) * inv;
-      }
-      nr[3] = real(1.5) / inv;
-    }
-  }
-  __syncthreads();
-  constexpr int EW = T / (kFluxThreads / 32);  // elements per warp
-  constexpr int UE = NF <= 4 ? EW : 1;                 // of which in flight together
-#pragma unroll 1
-  for (int it = lane; it < ITEMS; it += 32) {
-    const int f = it / Nfp, a = it - f * Nfp;
-    int io = fidx[it];
-    if constexpr (kChecked) {
-      if (io >= Np) {
-        oob = true;
-        io = 0;
-      }
-    }
-#pragma unroll 1
-    for (int j0 = 0; j0 < EW; j0 += UE) {
-      real own[UE][NF], nbv[UE][NF];
-      bool wall[UE];
-#pragma unroll
-      for (int u = 0; u < UE; ++u) {
-        const int e = warp * EW + j0 + u;
-        const int c = e < ne ? CS[e * 4 + f] : -1;
-        wall[u] = c < 0;
-        const real* src = P.qin + size_t(e0 + (e < ne ? e : 0)) * NF * Np + io;
-#pragma unroll
-        for (int k = 0; k < NF; ++k) own[u][k] = src[k * Np];
-        if (c >= 0) {
-          const int64_t nb = int64_t(c >> 5);
-          if constexpr (kChecked) {
-            if (nb >= P.G || (c & 7) >= 6) {
-              oob = true;
-              wall[u] = true;
-              continue;
-            }
-          }
-          const int ni = nidx[(((c >> 3) & 3) * 6 + (c & 7)) * Nfp + a];
-          if constexpr (kChecked) {
-            if (ni >= Np) {
-              oob = true;
-              wall[u] = true;
-              continue;
-            }
-          }
-          const real* nsrc = P.qin + size_t(nb) * NF * Np + ni;
-#pragma unroll
-          for (int k = 0; k < NF; ++k) nbv[u][k] = nsrc[k * Np];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < UE; ++u) {
-        const int e = warp * EW + j0 + u;
-        if (e >= ne) continue;
-        if (wall[u]) mirror(own[u], nbv[u]);
-        real out[NQ];
-        flux(NRM + (e * 4 + f) * 4, own[u], nbv[u], out);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) FL[(q * ITEMS + it) * ST + e] = out[q];
-      }
-    }
-  }
-  __syncthreads();
-  real* dst = P.flux + size_t(e0 / 32) * 32 * NQ * ITEMS + e0 % 32;
-  for (int x = tid; x < NQ * ITEMS * T; x += kFluxThreads) {
-    const int r = x / T, e = x % T;
-    if (e < ne) dst[size_t(r) * 32 + e] = FL[r * ST + e];
-  }
-  if constexpr (kChecked) {
-    if (oob) atomicOr(P.status, 2u);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// field tasks
-
-// grad lambda_0..3 and 1 / |grad lambda_f| of the lane's element
-// (LaneGeom::load: rows of the warp's block of kLaneGeom x 32 values)
-template <typename real>
-struct LaneGeom {
-  real g[4][3], inv[4];
-  __device__ __forceinline__ void load(const real* __restrict__ geom, int64_t e0, int lane) {
-    const real* p = geom + size_t(e0 / 32) * 32 * kLaneGeom + lane;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-#pragma unroll
-      for (int m = 1; m < 4; ++m) g[m][d] = p[(3 * (m - 1) + d) * 32];
-      g[0][d] = -g[1][d] - g[2][d] - g[3][d];
-    }
-#pragma unroll
-    for (int f = 0; f < 4; ++f) inv[f] = p[(9 + f) * 32];
-  }
-};
 
 // component d of the gradient of lambda_m
 template <typename real>
@@ -341,90 +173,6 @@ struct FieldRhs {
   }
 };
 
-// The lane's flux q on face f (fl: the warp's [NQ][4][Nfp][32] block at the lane).
-template <int N, int f, typename real>
-__device__ __forceinline__ void load_flux(const real* __restrict__ fl, int q, real (&F)[np2(N)]) {
-  const real* src = fl + (q * 4 + f) * np2(N) * 32;
-#pragma unroll
-  for (int i = 0; i < np2(N); ++i) F[i] = src[i * 32];
-}
-
-// The task's flux on face f, sum over its lift terms of n_d F_q (F holds the
-// first term's flux), lifted into the lane's right-hand side.
-template <typename Phys, int N, int f, typename real>
-__device__ __forceinline__ void lift_face(const TaskDesc& td, const real* __restrict__ fl, const LaneGeom<real>& gm,
-                                          real (&F)[np2(N)], real (&r)[np3(N)]) {
-  constexpr int Nfp = np2(N);
-  real w = td.l[0].dir >= 0 ? -pick(gm.g[f], td.l[0].dir) * gm.inv[f] : real(1);
-  if constexpr (Phys::MAXL > 1) {
-    if (td.nl > 1) {
-#pragma unroll
-      for (int i = 0; i < Nfp; ++i) F[i] *= w;
-      w = real(1);
-#pragma unroll 1
-      for (int t = 1; t < td.nl; ++t) {
-        const Term tm = t == 1 ? td.l[1] : td.l[2];
-        const real wt = tm.dir >= 0 ? -pick(gm.g[f], tm.dir) * gm.inv[f] : real(1);
-        const real* src = fl + (tm.what * 4 + f) * Nfp * 32;
-#pragma unroll
-        for (int i = 0; i < Nfp; ++i) F[i] = fma(wt, src[i * 32], F[i]);
-      }
-    }
-  }
-  FieldRhs<N, real>::template lift<f>(r, F, w);
-}
-
-// Right-hand side r of field task td, lane = element; gm: the lane's
-// geometry, cols: the warp's columns (stride S) for the staged fields.
-// Loads are issued one step ahead: the first flux before the staging, each
-// term's field (where the registers allow) and each face's flux during the
-// work on the one before.
-template <typename Phys, int N, typename real, int S>
-__device__ __forceinline__ void field_rhs(const TaskDesc& td, const real* __restrict__ qin,
-                                          const real* __restrict__ fluxes, int64_t e0, int ne, int lane, real* cols,
-                                          const LaneGeom<real>& gm, real (&r)[np3(N)]) {
-  using R = FieldRhs<N, real>;
-  using Tile = WarpTile<np3(N), real>;
-  constexpr int Np = R::Np, Nfp = R::Nfp, NF = Phys::NF, ES = NF * Np;
-  constexpr bool AHEAD = Tile::IT * Tile::W * int(sizeof(real)) <= 4 * 100;
-  constexpr int U = Tile::IT < 16 ? Tile::IT : 16;
-  const real* col = cols + lane * S;
-  const real* q0 = qin + size_t(e0) * ES;
-  const real* fl = fluxes + size_t(e0 / 32) * 32 * Phys::NQ * 4 * Nfp + lane;
-  typename Tile::Held held;
-  if constexpr (AHEAD) Tile::template hold<ES>(held, q0 + td.d[0].what * Np, lane, ne);
-  real F3[Nfp], F2[Nfp], F1[Nfp], F0[Nfp];
-  load_flux<N, 3>(fl, td.l[0].what, F3);
-  real v1[R::Nm1p];
-#pragma unroll
-  for (int i = 0; i < R::Nm1p; ++i) v1[i] = real(0);
-#pragma unroll 1
-  for (int t = 0; t < td.nd; ++t) {
-    const Term tm = t == 0 ? td.d[0] : t == 1 ? td.d[1] : td.d[2];
-    if (t > 0) __syncwarp();
-    if constexpr (AHEAD) {
-      Tile::template put<S>(held, cols, lane, ne);
-      if (t + 1 < td.nd) Tile::template hold<ES>(held, q0 + (t == 0 ? td.d[1].what : td.d[2].what) * Np, lane, ne);
-    } else {
-      Tile::template stage<ES, S, U>(cols, q0 + tm.what * Np, lane, ne);
-    }
-    __syncwarp();
-    real w[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) w[m] = real(Phys::SIGN) * pick(gm.g[m], tm.dir);
-    R::add_term(v1, col, w);
-  }
-  __syncwarp();  // the columns are free
-  R::elevate_all(v1, r);
-  load_flux<N, 2>(fl, td.l[0].what, F2);
-  lift_face<Phys, N, 3>(td, fl, gm, F3, r);
-  load_flux<N, 1>(fl, td.l[0].what, F1);
-  lift_face<Phys, N, 2>(td, fl, gm, F2, r);
-  load_flux<N, 0>(fl, td.l[0].what, F0);
-  lift_face<Phys, N, 1>(td, fl, gm, F1, r);
-  lift_face<Phys, N, 0>(td, fl, gm, F0, r);
-}
-
 // Power coefficients c_beta / beta! of the lane's degree-M weight, times s.
 // The weights of the warp's elements (ES values apart) are loaded ahead
 // (WeightTile::hold) and transposed through the free columns.
@@ -484,13 +232,6 @@ __device__ __forceinline__ void put_column(real* col, const real (&r)[Np]) {
 #pragma unroll
   for (int i = 0; i < Np; ++i) col[i] = r[i];
 }
-
-template <int N, typename real>
-using FieldShape = LaneShape<(np3(N) > np3(kMaxM) ? np3(N) : np3(kMaxM)), real, (N >= 6 ? 8 : 4)>;
-// CTAs per SM that the field kernels' registers have to allow: as many as fit
-// without spills at M <= 2
-template <int N>
-constexpr int kFieldCtas = N == 1 ? 10 : N == 2 ? 8 : N == 3 ? 6 : N == 4 ? 4 : N == 5 ? 3 : 1;
 
 // RK update of field fld (of NF) of the warp's elements from the columns:
 // res = a res + dt rhs, q_out = q_in + b res.
