@@ -104,6 +104,7 @@ EXPORTS = {
     "bbw_elastic_advance": (_int, [_p, _d, _d, _dp, _i64p]),
     "bbw_elastic_sync": (_int, [_p]),
     "bbw_elastic_get_time": (_int, [_p, _dp, _i64p]),
+    "bbw_internal_lane_min": (_i64, [_int, _int, _int, _int]),  # not in the header
     # include/bbw_nn.h: the surrogate's kernels
     "bbw_nn_gemm": (_int, [_int, _int, _int, _p, _int, C.c_longlong, _int, _p, _int, C.c_longlong, _int, _p, _int,
                            C.c_longlong, _int, C.c_float, C.c_float, _p, _p, _int, _int, _p]),

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "bbw_common.h"
+#include "bbw_elastic_ops.h"
 #include "bbw_ops.h"
 #include "bbw_stage.cuh"
 #include "bbwadg.h"
@@ -770,7 +771,7 @@ bbw_status bbw::create_solver(int64_t nverts, const double* vxyz, int64_t K, con
   }
   int team = 0, gpc = 1;
   s->ops->launch_shape(M, precision == 64, &team, &s->V, &gpc);
-  s->lane = s->ops->use_lane(M, precision == 64, K);
+  s->lane = K >= s->ops->lane_min(M, precision == 64);
   if (s->lane) s->V = 1;
   s->G = (K + s->V - 1) / s->V;
   const int64_t tiles = (s->G + gpc - 1) / gpc;
@@ -1062,6 +1063,13 @@ bbw_status bbw_validate_tables(int N, int M, int precision) {
   const char* msg = bbw::ops_for(N)->check_tables(M, precision == 64, cj);
   if (msg) return fail(BBW_ERR_ARG, std::string("operator table check failed: ") + msg);
   return BBW_OK;
+}
+
+// Not part of the interface (tests choose their sizes by it): the elements from
+// which on a solver runs the kernels with one element per lane, INT64_MAX if none
+// does. Host only; arguments in the ranges of bbw_create and bbw_elastic_create.
+int64_t bbw_internal_lane_min(int elastic, int N, int M, int precision) {
+  return elastic ? bbw::elastic_ops_for(N)->lane_min(M, precision == 64) : bbw::ops_for(N)->lane_min(M, precision == 64);
 }
 
 bbw_status bbw_lsrk_coeffs(double* a, double* b, double* c) {

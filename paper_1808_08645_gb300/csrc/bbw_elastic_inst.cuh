@@ -43,15 +43,28 @@ auto edispatch(int M, bool dbl, F&& f) {
 
 // FP32, N = 2..7: the kernels with one element per lane for solvers of at
 // least kELaneMin elements, otherwise the team kernel: below that the lane
-// kernels' two more launches and their few, long warps cost more than they save.
-// Stage times in us, lane / team, M = 2, at 2,058 / 4,374 / 24,576 elements:
-// N = 2 29/21, 29/21, 44/72; N = 3 31/21, 36/27, 71/133; N = 4 42/31, 45/58,
-// 122/191; N = 5 36/35, 41/66, 156/348; N = 6 56/49, 71/90, 274/468; N = 7
-// 76/99, 124/146, 458/744. The projections are fused up to N = 5, where their
-// levels fit the register file.
+// kernels' two or three more launches and their few, long warps cost more than
+// they save. The team kernel's time jumps where an SM gets one more CTA (its
+// elements x 152 SMs: N = 2, 3 every 2,432 elements a CTA, up to four CTAs;
+// N = 4 3,648, N = 5 and 6 2,432, N = 7 1,672) and the lane kernels' rises
+// evenly, so the constants lie behind the step from which on they are nowhere
+// slower (every 3.5 % of size measured, M = 0..3; lane / team before and behind):
+//   N = 2  M = 0: 1.54 below 9,728, 1.05 to 1.09 up to 19,456, 0.88 above; M = 1: 1.40, 0.96;
+//          M = 2: 1.22, 0.76; M = 3: 1.03 below 4,864, 0.95 up to 9,728, 0.54 above
+//   N = 3  M = 0: 1.32 below 7,296, 0.92; M = 1: 1.20, 0.84; M = 2, 3: 1.4 and 1.03 below 4,864, 0.82 and 0.58
+//   N = 4  1.06 to 1.7 below 3,648, 0.58 to 0.92; M = 0: 1.00 to 1.11 up to 7,296, 0.79 above
+//   N = 5  0.91 to 1.29 below 2,432, 0.50 to 0.80       N = 6  0.98 to 1.5 below 2,432, 0.55 to 0.87;
+//          M = 0 1.02 between 4,086 and 4,864           N = 7  1.4 to 1.66 below 1,672, 0.75 to 0.90
+// The projections are fused up to N = 5, where their levels fit the register file.
 template <typename real>
 constexpr bool kELane = sizeof(real) == 4 && kN >= 2 && kN <= 7;
-constexpr int64_t kELaneMin = kN <= 3 ? 7000 : kN == 4 ? 4000 : kN == 5 ? 3000 : kN == 6 ? 4000 : 1500;
+template <int M>
+constexpr int64_t kELaneMin = kN == 2   ? (M == 0 ? 19500 : M == 3 ? 7000 : 9800)
+                              : kN == 3 ? (M <= 1 ? 7300 : 7000)
+                              : kN == 4 ? (M == 0 ? 7300 : 4000)
+                              : kN == 5 ? 3000
+                              : kN == 6 ? (M == 0 ? 4900 : 4000)
+                                        : 1700;
 constexpr bool kEFused = kN <= 5;
 template <int M, typename real>
 using EFCfg = FieldShape<kN, real>;
@@ -117,12 +130,16 @@ cudaError_t elaunch(int M, bool dbl, const void* params, int grid, cudaStream_t 
   });
 }
 
+int64_t elane_min(int M, bool dbl) {
+  return edispatch(M, dbl, [&]<int MM, typename real>() { return kELane<real> ? kELaneMin<MM> : INT64_MAX; });
+}
+
 // Elements per group and scratch of a solver of K elements; see ElasticOps.
 int elayout(int M, bool dbl, int64_t K, size_t* flux, size_t* trace) {
   return edispatch(M, dbl, [&]<int MM, typename real>() {
     *flux = *trace = 0;
     if constexpr (kELane<real>) {
-      if (K >= kELaneMin) {
+      if (K >= kELaneMin<MM>) {
         *flux = flux_values(K, np2(kN));
         *trace = size_t(K) * np3(kN);
         return 1;
@@ -153,7 +170,7 @@ void eshape(int M, bool dbl, int* team, int* width, int* groups) {
 #define BBW_ECAT2(a, b) a##b
 #define BBW_ECAT(a, b) BBW_ECAT2(a, b)
 const ElasticOps& BBW_ECAT(elastic_ops_n, BBW_N)() {
-  static const ElasticOps ops = {&eprepare, &elaunch, &eshape, &elayout, &escale};
+  static const ElasticOps ops = {&eprepare, &elaunch, &eshape, &elayout, &elane_min, &escale};
   return ops;
 }
 

@@ -21,6 +21,8 @@ struct ElasticOps {
   // elements per group of the layout of a solver of K elements, and its scratch
   // in values: face fluxes and the trace (0: the team kernel, which uses none)
   int (*layout)(int M, bool dbl, int64_t K, size_t* flux, size_t* trace);
+  // elements from which on layout takes the kernels with one element per lane
+  int64_t (*lane_min)(int M, bool dbl);
   // constants cs[N + 1] of the projection kernels from the N + 1 constants c_j
   void (*projection_scale)(int M, const double* cj, double* cs);
 };

@@ -31,9 +31,9 @@ struct KernelOps {
   const char* (*check_tables)(int M, bool dbl, const double* cj);
   // launch the adjoint stage's pre-kernel; params points to LaneAdjPreParams<float|double>
   cudaError_t (*launch_adj_pre)(int M, bool dbl, const void* params, int grid, cudaStream_t s);
-  // whether a solver of K elements runs the tile kernels (bbw_tile.cuh; the
+  // elements from which on a solver runs the tile kernels (bbw_tile.cuh; the
   // launch entries do so when the parameters' lane is set)
-  bool (*use_lane)(int M, bool dbl, int64_t K);
+  int64_t (*lane_min)(int M, bool dbl);
 };
 
 const KernelOps& ops_n1();

@@ -48,22 +48,37 @@ constexpr auto adj_pre_fn() {
 // The tile kernels (bbw_tile.cuh) run solvers of at least kLaneMin elements,
 // N <= 6 in FP32 and N <= 5 in FP64; the team kernels (bbw_stage.cuh) the rest
 // (the same bits either way). A tile has 32 elements, so small meshes leave
-// SMs idle, and a warp's chain of work is longer than a team's. Stage times in
-// us, tile / team, M = 2, at 384 / 4,374 / 24,576 / 82,944 elements, FP32:
-//   N = 1  6.3/6.6, 7.3/8.3, 10/10, 20/27     N = 2  10/8.3, 10/8.4, 15/21, 34/47
-//   N = 3  12/10, 13/11, 20/31, 51/84         N = 4  17/20, 18/21, 42/51, 110/146
-//   N = 5  19/27, 20/29, 44/75, 145/219       N = 6  27/21, 29/21, 100/105, 270/302
-// (10,368 elements: N = 2 12.0/12.5, N = 3 14/18, N = 6 56/54; N = 7 at 82,944
-// 456/412, and N >= 8 does not fit). N = 6 gains least, and at M = 0 nothing
-// at 24,576 (92/91) and 256/262 at 82,944; a last wave in between can cost 5 %,
-// so it switches above those. FP64 at 384 / 6,000 / 16,464 elements:
-//   N = 1  18/27, 23/29, 37/47      N = 2  38/35, 53/62, 89/121    N = 3  60/37, 91/96, 156/245
-//   N = 4  111/120, 152/236, 299/466               N = 5  187/94, 267/275, 448/636
+// SMs idle, and a warp's chain of work is longer than a team's. Both times rise
+// in steps, at the sizes where an SM gets one more CTA (tile: multiples of 32 x
+// 152 = 4,864 elements; team: of its CTA's elements x 152), so their ratio
+// jumps there, and the constants lie at the steps from which on the tile kernel
+// is nowhere slower (every 3 to 5 % of size measured, M = 0..3; tile / team):
+//   FP32, N = 1  M = 0, 1: 1.00 below 4,900, 1.26 up to 9,728 (both sizes one
+//                step higher: 7.9 us against 6.2 a stage), 0.95 to 1.00 above, and
+//                at M = 0 again 1.03 to 1.14 between 34,800 and 57,000;
+//                M = 2, 3: below 1 everywhere (4,374 elements: 0.78)
+//         N = 2  1.00 to 1.25 below, 0.91 to 0.97 at 9,867
+//         N = 3  1.0 to 1.2 below 4,864, 0.86 to 0.97 above, 0.70 to 0.85 from 9,757
+//         N = 4  0.79 to 0.98 below 9,728, 0.55 to 0.85 above
+//         N = 5  0.60 to 0.75 below, 0.38 to 0.78 above
+//         N = 6  1.6 to 1.95 below 4,864, 1.05 to 1.2 below 14,600, then by steps
+//                0.82 to 1.05, and 0.80 to 0.99 from 65,000
+//   FP64, N = 1  0.50 to 0.94       N = 2  0.98 to 1.10 below 4,864, 0.76 to 0.89 above
+//         N = 3  up to 1.7 below 2,432, 0.91 to 1.01 up to 4,864, 0.91 to 0.96 above
+//         N = 4  0.55 to 0.98       N = 5  1.01 to 2.1 below, 0.93 to 0.97 above
+// Us a stage, M = 2, 82,944 elements, FP32, tile / team: N = 1 21/27, 2 33/46,
+// 3 50/82, 4 110/146, 5 142/219, 6 270/302; N = 7 456/412, and N >= 8 does not
+// fit the registers.
 template <typename real>
 constexpr bool kLane = kN <= (sizeof(real) == 4 ? 6 : 5);
-template <typename real>
-constexpr int64_t kLaneMin = sizeof(real) == 4 ? (kN == 2 ? 10000 : kN == 3 ? 9000 : kN == 6 ? 80000 : 0)
-                                               : (kN == 2 || kN == 3 ? 5000 : kN == 5 ? 6000 : 0);
+template <int M, typename real>
+constexpr int64_t kLaneMin = sizeof(real) == 4
+                                 ? (kN == 1 ? (M == 0 ? 59000 : M == 1 ? 9800 : 0)
+                                    : kN == 2 ? 10000
+                                    : kN == 3 ? 9000
+                                    : kN == 6 ? 80000
+                                              : 0)
+                                 : (kN == 2 || kN == 3 ? 5000 : kN == 5 ? 6000 : 0);
 // The projection of p runs in the tile kernel where its levels fit the
 // registers (N <= 5, FP64 4); at N = 6 one warp of four would work on it for
 // longer than the rest of the tile takes (291 us fused, 270 apart).
@@ -234,8 +249,8 @@ cudaError_t launch_adj_pre(int M, bool dbl, const void* params, int grid, cudaSt
   });
 }
 
-bool use_lane(int M, bool dbl, int64_t K) {
-  return dispatch(M, dbl, [&]<int MM, typename real>() { return kLane<real> && K >= kLaneMin<real>; });
+int64_t lane_min(int M, bool dbl) {
+  return dispatch(M, dbl, [&]<int MM, typename real>() { return kLane<real> ? kLaneMin<MM, real> : INT64_MAX; });
 }
 
 }  // namespace
@@ -245,7 +260,7 @@ bool use_lane(int M, bool dbl, int64_t K) {
 const KernelOps& BBW_CAT(ops_n, BBW_N)() {
   static const KernelOps ops = {&tables_size,  &build,          &face_maps,    &prepare,
                                 &launch_stage, &launch_wadg,    &launch_shape, &launch_spatial,
-                                &check_tables, &launch_adj_pre, &use_lane};
+                                &check_tables, &launch_adj_pre, &lane_min};
   return ops;
 }
 

@@ -51,3 +51,23 @@ def test_elastic_stage(N, n, M, s):
     q, r = (rounded(rng, -1, 1, (9, len(e), Np)) for _ in range(2))
     a, b = (stage(p, v, e, N, M, media, q, r, s) for p in (B.F32, B.F64))
     assert rel_l2(a, b) <= 1e-5
+
+
+@pytest.mark.parametrize("N,M,n", [(2, 0, 15), (2, 1, 12), (2, 2, 12), (3, 0, 11), (4, 0, 11), (5, 0, 9), (6, 0, 10), (7, 0, 7)])
+def test_elastic_step(N, M, n):
+    """Constant media, and the media degrees of N = 2 above their own switching sizes; five stages in turn, whose error is at
+    most the five stages', each below the stage's bound."""
+    v, e = mesh(n)
+    assert len(e) >= B.lib().bbw_internal_lane_min(1, N, M, 32)
+    rng = np.random.default_rng(300 * N + M)
+    Np, Mp = (N + 1) * (N + 2) * (N + 3) // 6, (M + 1) * (M + 2) * (M + 3) // 6
+    media = [rounded(rng, 0.5, 1.5, (len(e), Mp)) for _ in range(3)]
+    q = rounded(rng, -1, 1, (9, len(e), Np))
+    out = []
+    for prec in (B.F32, B.F64):
+        with B.ElasticSolver(v, e, N, M, prec) as solver:
+            solver.set_media(*media)
+            solver.set_state(q)
+            solver.step(1e-4, 1)
+            out.append(solver.get_state()[0])
+    assert rel_l2(*out) <= 5e-5
