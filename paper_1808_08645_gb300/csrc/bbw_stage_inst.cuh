@@ -79,6 +79,9 @@ constexpr int64_t kLaneMin = sizeof(real) == 4
                                     : kN == 6 ? 80000
                                               : 0)
                                  : (kN == 2 || kN == 3 ? 5000 : kN == 5 ? 6000 : 0);
+// The team kernels of the stage exist for solvers below that size only.
+template <int M, typename real>
+constexpr bool kTeam = !kLane<real> || kLaneMin<M, real> > 0;
 // The projection of p runs in the tile kernel where its levels fit the
 // registers (N <= 5, FP64 4); at N = 6 one warp of four would work on it for
 // longer than the rest of the tile takes (291 us fused, 270 apart).
@@ -149,12 +152,17 @@ cudaError_t allow_smem(K kernel, int bytes) {
 cudaError_t prepare(int M, bool dbl, int* per_sm_stage, int* per_sm_wadg) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    auto ks = stage_fn<MM, real>();
     auto kw = wadg_fn<MM, real>();
-    cudaError_t err = allow_smem(ks, C::SMEM);
-    if (err == cudaSuccess) err = allow_smem(kw, C::SMEM);
-    if (err == cudaSuccess) err = allow_smem(spatial_fn<MM, real>(), C::SMEM);
-    if (err == cudaSuccess) err = allow_smem(adj_pre_fn<MM, real>(), C::SMEM);
+    *per_sm_stage = 1;
+    cudaError_t err = allow_smem(kw, C::SMEM);
+    if constexpr (kTeam<MM, real>) {
+      auto ks = stage_fn<MM, real>();
+      if (err == cudaSuccess) err = allow_smem(ks, C::SMEM);
+      if (err == cudaSuccess) err = allow_smem(spatial_fn<MM, real>(), C::SMEM);
+      if (err == cudaSuccess) err = allow_smem(adj_pre_fn<MM, real>(), C::SMEM);
+      if (err == cudaSuccess)
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm_stage, ks, C::THREADS, C::SMEM);
+    }
     if constexpr (kLane<real>) {
       using PC = ProjectShape<kN, MM, real>;
       if (err == cudaSuccess) err = allow_smem(tile_fn<MM, real, kStageMode<real>>(), TileCfg<kN, real>::SMEM);
@@ -163,8 +171,6 @@ cudaError_t prepare(int M, bool dbl, int* per_sm_stage, int* per_sm_wadg) {
       if constexpr (!kFuseProjection<real>)
         if (err == cudaSuccess) err = allow_smem(acoustic_project_kernel<kN, MM, real>, PC::SMEM);
     }
-    if (err != cudaSuccess) return err;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm_stage, ks, C::THREADS, C::SMEM);
     if (err != cudaSuccess) return err;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm_wadg, kw, C::THREADS, C::SMEM);
   });
@@ -191,7 +197,7 @@ cudaError_t launch_stage(int M, bool dbl, const void* params, int grid, cudaStre
     using C = Cfg<MM, real>;
     const auto& P = *static_cast<const LaneStageParams<real>*>(params);
     if constexpr (kLane<real>) {
-      if (P.lane) {
+      if (P.lane || !kTeam<MM, real>) {
         launch_tiles<MM, real, kStageMode<real>>(P, s);
         if constexpr (!kFuseProjection<real>) {
           using PC = ProjectShape<kN, MM, real>;
@@ -202,7 +208,7 @@ cudaError_t launch_stage(int M, bool dbl, const void* params, int grid, cudaStre
         return cudaGetLastError();
       }
     }
-    stage_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
+    if constexpr (kTeam<MM, real>) stage_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
     return cudaGetLastError();
   });
 }
@@ -212,12 +218,12 @@ cudaError_t launch_spatial(int M, bool dbl, const void* params, int grid, cudaSt
     using C = Cfg<MM, real>;
     const auto& P = *static_cast<const LaneStageParams<real>*>(params);
     if constexpr (kLane<real>) {
-      if (P.lane) {
+      if (P.lane || !kTeam<MM, real>) {
         launch_tiles<MM, real, kSpatial>(P, s);
         return cudaGetLastError();
       }
     }
-    spatial_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
+    if constexpr (kTeam<MM, real>) spatial_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
     return cudaGetLastError();
   });
 }
@@ -236,7 +242,7 @@ cudaError_t launch_adj_pre(int M, bool dbl, const void* params, int grid, cudaSt
     using C = Cfg<MM, real>;
     const auto& P = *static_cast<const LaneAdjPreParams<real>*>(params);
     if constexpr (kLane<real>) {
-      if (P.lane) {
+      if (P.lane || !kTeam<MM, real>) {
         using PC = ProjectShape<kN, MM, real>;
         const int w = lane_warps<PC>(P.G);
         lane_adj_pre_kernel<kN, MM, real>
@@ -244,7 +250,7 @@ cudaError_t launch_adj_pre(int M, bool dbl, const void* params, int grid, cudaSt
         return cudaGetLastError();
       }
     }
-    adj_pre_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
+    if constexpr (kTeam<MM, real>) adj_pre_fn<MM, real>()<<<grid, C::THREADS, C::SMEM, s>>>(P);
     return cudaGetLastError();
   });
 }
