@@ -311,10 +311,10 @@ __device__ __forceinline__ void field_rhs(const TaskDesc& td, const real* __rest
 
 template <int N, typename real>
 using FieldShape = LaneShape<(np3(N) > np3(kMaxM) ? np3(N) : np3(kMaxM)), real, (N >= 6 ? 8 : 4)>;
-// CTAs per SM that the field kernels' registers have to allow: as many as fit
-// without spills at M <= 2
+// CTAs per SM that the field kernels' registers have to allow. Stack at
+// M <= 2: 8 to 72 bytes at N = 2, 32 to 112 at N = 3, none to 16 above
 template <int N>
-constexpr int kFieldCtas = N == 2 ? 8 : N == 3 ? 6 : N == 4 ? 4 : N == 5 ? 3 : 1;
+constexpr int kFieldCtas = N == 2 ? 8 : N == 3 ? 6 : N == 4 ? 4 : N == 5 ? 2 : 1;
 
 // The projected right-hand side of a field in the columns -> its RK update;
 // the trace task stores its projection instead. task as in elastic_task.
@@ -355,7 +355,7 @@ __device__ __forceinline__ int elastic_weight(int task) { return task < 3 ? 0 : 
 // launch are TRACE ? {trace, v_x, v_y, v_z} : the six stresses. Otherwise the
 // brackets go to q_out and P.trace for elastic_project_kernel.
 template <int N, int M, typename real, bool FUSED, bool TRACE>
-__global__ void __launch_bounds__(FieldShape<N, real>::THREADS, N == 5 ? 2 : kFieldCtas<N>)
+__global__ void __launch_bounds__(FieldShape<N, real>::THREADS, kFieldCtas<N>)
     elastic_field_kernel(const LaneElasticParams<real> P) {
   using C = FieldShape<N, real>;
   using Tile = WarpTile<np3(N), real>;
@@ -402,7 +402,8 @@ __global__ void __launch_bounds__(FieldShape<N, real>::THREADS, N == 5 ? 2 : kFi
 
 // Projections and RK updates from the brackets in q_out and P.trace, tasks per
 // launch as in the fused elastic_field_kernel. A warp reads its whole bracket
-// before it writes the field there.
+// before it writes the field there. At N = 7 the levels do not fit the 255
+// registers: 136 to 280 bytes of stack.
 template <int N, int M, typename real, bool TRACE>
 __global__ void __launch_bounds__(ProjectShape<N, M, real>::THREADS)
     elastic_project_kernel(const LaneElasticParams<real> P) {

@@ -20,10 +20,10 @@
 // word), and in FP64 the double-precision pipe, on which the conversions of
 // the integer weights cost as much as the products; here a stage needs about
 // half the warp instructions per element and no conversions. What bounds it
-// now (N = 5, 82,944 elements: 145 us against 219) is latency: 10 to 12 warps
-// per SM at 0.33 instructions per scheduler and cycle, waiting in turn for the
-// staged field, the neighbour gather and the RK operands; L1 wavefronts 37 %,
-// DRAM 1.8 TB/s. Separate kernels for the fluxes and the fields (more warps in
+// now (N = 5, 82,944 elements: 142 us against 219) is latency: 9.7 of 12 warps
+// per SM at 0.33 instructions per scheduler and cycle, waiting for the staged
+// field, the neighbour gather and the RK operands in turn and for instructions;
+// L1 wavefronts 38 % of their peak, DRAM 21 %. Separate kernels for the fluxes and the fields (more warps in
 // flight, the fluxes through L2) took 150 us.
 // The operations and their order are those of stage_kernel (bbw_stage.cuh):
 // the results are the same bits, so the two can be chosen by size.
@@ -52,7 +52,9 @@ struct TileCfg {
   static constexpr int REALS = 4 * 32 * S + 2 * ITEMS * FS + 512 + 288 + 128;
   static constexpr int SMEM = (REALS * int(sizeof(real)) + 512 + 56 * Nfp + 15) / 16 * 16;
   static constexpr int THREADS = 128;
-  // CTAs per SM that the registers have to allow (no spills at M <= 2)
+  // CTAs per SM that the registers have to allow. Stack of the fused kernel:
+  // FP32 none but 8 bytes at N = 3 (M = 3: 40); FP64 at N = 4 72 to 88 bytes at
+  // M <= 1, 528 at M = 2, 1,240 at M = 3, and 360 at N = M = 3
   static constexpr int CTAS = sizeof(real) == 8 ? (N <= 4 ? 4 : 2) : N <= 2 ? 8 : N == 3 ? 6 : N == 4 ? 4 : N == 5 ? 3 : 2;
 };
 
