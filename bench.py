@@ -285,7 +285,7 @@ def run_gpu(args):
                          "algorithmic_bytes_per_launch": algorithmic_bytes_per_element(top, M) * K,
                          "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback"},
             "e2e": e2e,
-            "gpu_launches": 5 * len(Ns) * args.steps,
+            "gpu_launches": 5 * sum(stage_launches(N, K, M) for N in Ns) * args.steps,
             "clocks": clk,
         }
         if not args.no_cpu_baseline:
@@ -346,12 +346,24 @@ def run_e2e(solvers, host_q0, Ns, dts, K, steps, stream):
                     "bytes per step amortised over the run"}
 
 
+def stage_launches(N: int, K: int, M: int, elastic: bool = False) -> int:
+    """Kernels that one FP32 stage of a solver (or bucket) of K elements launches. The team kernels are one; of the kernels
+    with one element per lane the acoustic ones are one up to N = 5 and two with the projection apart, the elastic ones
+    three (fluxes, trace and velocities, stresses) and four (the projections apart)."""
+    from paper_1808_08645_gb300 import binding as B
+    if K < B.lib().bbw_internal_lane_min(int(elastic), N, M, 32):
+        return 1
+    return (3 if N <= 5 else 4) if elastic else (1 if N <= 5 else 2)
+
+
 # the sources that decide the stage kernel's memory traffic: the kernel and
 # its tables, and the host code that lays out and orders the elements
-KERNEL_SOURCES = ("bbw_stage.cuh", "bbw_common.h", "bbw_stage_inst.cuh", "bbw_api.cu")
-# the same for the elastic stage kernel
-ELASTIC_SOURCES = ("bbw_elastic.cuh", "bbw_stage.cuh", "bbw_common.h", "bbw_elastic_inst.cuh",
-                   "bbw_elastic.cu", "bbw_api.cu")
+LANE_SOURCES = ("bbw_lane.cuh", "bbw_project.cuh", "bbw_warp_tile.cuh")
+KERNEL_SOURCES = ("bbw_stage.cuh", "bbw_common.h", "bbw_stage_inst.cuh", "bbw_ops.h", "bbw_tile.cuh",
+                  *LANE_SOURCES, "bbw_api.cu")
+# the same for the elastic stage kernels
+ELASTIC_SOURCES = ("bbw_elastic.cuh", "bbw_stage.cuh", "bbw_common.h", "bbw_elastic_inst.cuh", "bbw_elastic_ops.h",
+                   "bbw_elastic_lane.cuh", *LANE_SOURCES, "bbw_elastic.cu", "bbw_api.cu")
 
 
 def sources_sha256(names) -> str:
@@ -579,6 +591,7 @@ def run_batched(args):
         qs, _ = s.get_state()
         err = max(err, float(np.linalg.norm(qb - qs) / max(np.linalg.norm(qs), 1e-300)))
     n, nbuckets, elements = batch.info()
+    stage_kernels = sum(stage_launches(N, sum(len(m[1]) for m, x in zip(meshes, Ns) if x == N), M) for N in set(Ns))
     for s in solos:
         s.close()
     to_T = _batched_to_time(batch, specs, meshes, Ns, dt, cfg, timed, max(args.steps, 20) * dt, B)
@@ -596,7 +609,8 @@ def run_batched(args):
                                f"common CFL dt", "buckets": nbuckets, "elements_with_padding": elements,
                    "l2": "inputs larger than L2 (tens of GB of state)"},
         "batched": {"dof_updates_per_s": value_b, "ms_per_step": ms_batch / args.steps,
-                    "launch": "one CUDA graph per step: 5 persistent stage launches per degree bucket",
+                    "launch": f"one CUDA graph per step: 5 stages of {stage_kernels} kernels over {nbuckets} degree "
+                              "buckets, and the step counter",
                     "schedule": {0: "concurrent branches, solo grids", 1: "buckets in sequence, solo grids",
                                  2: "concurrent branches, half grids",
                                  3: "concurrent branches, double grids"}.get(schedule, str(schedule)),
@@ -605,7 +619,7 @@ def run_batched(args):
                   "launch": "one solo solver per instance, bbw_step per instance, one after another"},
         "max_rel_l2_batched_vs_plain": err,
         "to_time_T": to_T,
-        "gpu_launches": 5 * nbuckets * args.steps + args.steps,
+        "gpu_launches": (5 * stage_kernels + 1) * args.steps,
         "setup_s": t_setup, "clocks": clocks,
     }
 
@@ -1046,7 +1060,7 @@ def run_elastic(args):
                 "d2h_bytes_per_step": d2h / e2e_steps,
                 "note": f"per degree: bbw_elastic_set_state from pinned host FP64, {e2e_steps} RK steps, "
                         "bbw_elastic_get_state into pinned host FP64"},
-        "gpu_launches": 5 * len(Ns) * args.steps,
+        "gpu_launches": 5 * sum(stage_launches(N, K, M, elastic=True) for N in Ns) * args.steps,
         "clocks": clk,
     }
     if not args.no_cpu_baseline:

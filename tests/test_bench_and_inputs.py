@@ -6,6 +6,7 @@ from __future__ import annotations
 import argparse
 import json
 import os
+import re
 import sys
 
 import numpy as np
@@ -150,3 +151,28 @@ def test_manufactured_forcing_makes_the_manufactured_solution_exact():
     ut = (u(x, t + h) - u(x, t - h)) / (2 * h)
     gp = np.stack([(p(x + h * np.eye(3)[i], t) - p(x - h * np.eye(3)[i], t)) / (2 * h) for i in range(3)], 1)
     assert np.allclose(ut + gp, 0.0, atol=1e-8)
+
+
+def test_traffic_sources_name_every_header_of_the_kernels():
+    """A capture counts as current only while no source that its kernel is compiled from has changed."""
+    csrc = os.path.join(ROOT, "paper_1808_08645_gb300", "csrc")
+
+    def headers(name, seen):
+        if name not in seen:
+            seen.add(name)
+            with open(os.path.join(csrc, name)) as fh:
+                for inc in re.findall(r'#include "(bbw_\w+\.cuh?)"', fh.read()):
+                    headers(inc, seen)
+        return seen
+
+    assert headers("bbw_stage_inst.cuh", set()) <= set(bench.KERNEL_SOURCES)
+    assert headers("bbw_elastic_inst.cuh", set()) <= set(bench.ELASTIC_SOURCES)
+
+
+def test_stage_launches_count_every_kernel():
+    from paper_1808_08645_gb300 import build
+    build.build()
+    K = 196608
+    assert [bench.stage_launches(N, K, 2) for N in range(1, 10)] == [1, 1, 1, 1, 1, 2, 1, 1, 1]
+    assert [bench.stage_launches(N, K, 2, elastic=True) for N in range(1, 10)] == [1, 3, 3, 3, 3, 4, 4, 1, 1]
+    assert bench.stage_launches(6, 384, 2) == bench.stage_launches(6, 384, 2, elastic=True) == 1
