@@ -23,9 +23,7 @@
 // one, in its order (product of factorial-scaled coefficients, Bernstein
 // reductions and elevations), so that its results are the same bits; it costs
 // one more multiplication per reduction and two more operations per elevation.
-// (Of degree 1 the team kernels' w = c v + (1/n) E w is one FMA, the compiler
-// having dropped the factor 1; so it is here. Written out there, it changed the
-// registers of wadg_kernel, which took up to 5 % longer.)
+// (Of degree 1 the team kernels' w = c v + (1/n) E w is one FMA; so it is here.)
 #pragma once
 
 #include <type_traits>

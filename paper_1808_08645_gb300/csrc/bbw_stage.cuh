@@ -283,10 +283,9 @@ __device__ __forceinline__ vec<real, V> vaxpy(const vec<real, V>& a, real w, con
   vfmas(r, w, b);
   return r;
 }
-// Products and differences that are not contracted into an FMA. |g|^2 and the
-// penalties, which the tile kernels (bbw_tile.cuh) repeat bit by bit, are written
-// with these and with fma, so that the rounding is the source's and not the
-// compiler's choice.
+// Products and differences that are not contracted into an FMA. What the tile
+// kernels (bbw_tile.cuh) repeat bit by bit is written with these and with fma,
+// so that the rounding is the source's and not the compiler's choice.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
@@ -552,8 +551,12 @@ __device__ __forceinline__ void wadg_group(const Tables<N, M, real>& tab, real* 
         if (s.w1 > 0) vfmas(acc, real(s.w1), vld<real, V>(X + (s.base - 1) * V));
         if (s.w2 > 0) vfmas(acc, real(s.w2), vld<real, V>(X + (s.base - s.dk) * V));
         if (s.w3 > 0) vfmas(acc, real(s.w3), vld<real, V>(X + (s.base - s.dl) * V));
-        w[r] = vmuls(c, lv[jl][r]);
-        vfmas(w[r], inv, acc);
+        if (n == 1) {  // 1/n = 1: one FMA
+          w[r] = vaxpy(acc, c, lv[jl][r]);
+        } else {
+          w[r] = vmuls(c, lv[jl][r]);
+          vfmas(w[r], inv, acc);
+        }
       }
     }
     if (jl > 0) {
