@@ -152,16 +152,21 @@ cudaError_t allow_smem(K kernel, int bytes) {
 cudaError_t prepare(int M, bool dbl, int* per_sm_stage, int* per_sm_wadg) {
   return dispatch(M, dbl, [&]<int MM, typename real>() {
     using C = Cfg<MM, real>;
-    auto kw = wadg_fn<MM, real>();
     *per_sm_stage = 1;
-    cudaError_t err = allow_smem(kw, C::SMEM);
+    cudaError_t err = cudaSuccess;
+    // (the stage kernel before the WADG kernel: instantiated the other way round,
+    // the latter is compiled to other registers, up to 5 % slower)
     if constexpr (kTeam<MM, real>) {
       auto ks = stage_fn<MM, real>();
-      if (err == cudaSuccess) err = allow_smem(ks, C::SMEM);
-      if (err == cudaSuccess) err = allow_smem(spatial_fn<MM, real>(), C::SMEM);
-      if (err == cudaSuccess) err = allow_smem(adj_pre_fn<MM, real>(), C::SMEM);
+      err = allow_smem(ks, C::SMEM);
       if (err == cudaSuccess)
         err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm_stage, ks, C::THREADS, C::SMEM);
+    }
+    auto kw = wadg_fn<MM, real>();
+    if (err == cudaSuccess) err = allow_smem(kw, C::SMEM);
+    if constexpr (kTeam<MM, real>) {
+      if (err == cudaSuccess) err = allow_smem(spatial_fn<MM, real>(), C::SMEM);
+      if (err == cudaSuccess) err = allow_smem(adj_pre_fn<MM, real>(), C::SMEM);
     }
     if constexpr (kLane<real>) {
       using PC = ProjectShape<kN, MM, real>;
