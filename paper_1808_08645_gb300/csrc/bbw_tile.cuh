@@ -53,7 +53,7 @@ struct TileCfg {
   static constexpr int SMEM = (REALS * int(sizeof(real)) + 512 + 56 * Nfp + 15) / 16 * 16;
   static constexpr int THREADS = 128;
   // CTAs per SM that the registers have to allow. Stack of the fused kernel:
-  // FP32 none but 8 bytes at N = 3 (M = 3: 40); FP64 at N = 4 72 to 88 bytes at
+  // FP32 none but 40 bytes at N = M = 3; FP64 at N = 4 72 to 88 bytes at
   // M <= 1, 528 at M = 2, 1,240 at M = 3, and 360 at N = M = 3
   static constexpr int CTAS = sizeof(real) == 8 ? (N <= 4 ? 4 : 2) : N <= 2 ? 8 : N == 3 ? 6 : N == 4 ? 4 : N == 5 ? 3 : 2;
 };
@@ -64,6 +64,26 @@ __device__ __forceinline__ bool all_finished(const StageParams<real>& P, int64_t
   if (!P.steps_group) return false;
   const int64_t step = P.step_dev ? *P.step_dev : P.step_host;
   return __all_sync(0xffffffffu, step >= P.steps_group[e0 + min(lane, ne - 1)]);
+}
+
+// q_out = q_in of a tile's ne elements, by the CTA. Out of line: inline, it cost
+// the tiles that are not finished up to 1 % (and N = 3 eight bytes of stack).
+template <int N, typename real>
+__device__ __noinline__ void carry_tile(const real* qin, real* qout, int64_t e0, int ne) {
+  constexpr int ES = 4 * np3(N);
+  const uint4* src = reinterpret_cast<const uint4*>(qin + size_t(e0) * ES);
+  uint4* dst = reinterpret_cast<uint4*>(qout + size_t(e0) * ES);
+  constexpr int ALL = 32 * ES * int(sizeof(real)) / 16, U = ALL < 12 * 128 ? (ALL + 127) / 128 : 12;
+  const int n = ALL / 32 * ne;
+  for (int i0 = threadIdx.x; i0 < n; i0 += 128 * U) {  // few CTAs fit an SM: many loads in flight in each
+    uint4 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i0 + 128 * u < n) x[u] = src[i0 + 128 * u];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i0 + 128 * u < n) dst[i0 + 128 * u] = x[u];
+  }
 }
 
 template <int N, int M, typename real, int MODE>
@@ -93,19 +113,7 @@ __global__ void __launch_bounds__(128, TileCfg<N, real>::CTAS)
     // its state over (every warp tests the same elements): N = 5, 63,888 finished
     // elements beside 48 live ones take 36 us a stage, and 124 when they are live.
     if (all_finished(P, e0, ne, lane)) {
-      const uint4* src = reinterpret_cast<const uint4*>(P.qin + size_t(e0) * ES);
-      uint4* dst = reinterpret_cast<uint4*>(P.qout + size_t(e0) * ES);
-      constexpr int ALL = 32 * ES * int(sizeof(real)) / 16, U = ALL < 12 * 128 ? (ALL + 127) / 128 : 12;
-      const int n = ALL / 32 * ne;
-      for (int i0 = tid; i0 < n; i0 += 128 * U) {  // few CTAs fit an SM: many loads in flight in each
-        uint4 x[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (i0 + 128 * u < n) x[u] = src[i0 + 128 * u];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (i0 + 128 * u < n) dst[i0 + 128 * u] = x[u];
-      }
+      carry_tile<N, real>(P.qin, P.qout, e0, ne);
       return;
     }
   }
